@@ -9,8 +9,6 @@ namespace segmg {
 
 constexpr int kCoarseThreads = 1024;
 constexpr int kWarpCoarseMax = 256;   // grids of at most this many cells are solved by one warp
-constexpr int kRegBand = 8;           // one warp keeps the band factor in registers up to this width
-                                      // (and at most 32 unknowns: one row per lane)
 
 // The threads that run the coarsest solve: one warp (no block barriers) or the whole block.
 template <int NT>
@@ -72,73 +70,199 @@ template <>
 __device__ __forceinline__ double rsqrt_of<double>(double s) { return 1.0 / sqrt(s); }
 
 // Banded Cholesky factorisation and solve of A x = b by one warp for N <= 32 unknowns and band
-// width bw <= kRegBand: lane r holds row r of the band (Lr[d] = A(r, r - d), then L(r, r - d);
-// Lr[0] keeps 1 / L(r, r)).  Column k's pivot and entries reach the other lanes by shuffles;
-// every element receives the same updates, in the same order, as in the shared-memory
-// factorisation.  The substitutions accumulate column by column.  Returns false (on every lane)
-// when a pivot is not positive; else lane r < N holds x(r) in xr.
-template <typename C>
-__device__ __forceinline__ bool warp_band_solve(const C *band, const C *b, int N, int bw, C &xr) {
+// width bw <= BAND.  Lane r owns row r and keeps a window of it in registers that slides with
+// the column k being eliminated: W[j] = A(r, k + j), j = 0 .. bw, for the rows k .. k + bw that
+// column k touches (the rows below are not in the window yet and wait with W[j] = A(r, r - bw + j)).
+// The pivot and the column's entries reach the other lanes by shuffles; the forward substitution
+// runs in the same loop; `band` (N x bw) holds the scaled columns for the backward one.  Every
+// element receives the updates of a right-looking factorisation in column order.  Returns false
+// (on every lane) when a pivot is not positive; else lane r < N holds x(r) in xr.
+// A lone warp's dependent chain sets the time: each loop body is a straight line with no branch, so
+// that its shuffles are in flight together (about 130 cycles a column; 940 with the whole band
+// unrolled per lane and the column's register found by comparisons).
+template <typename C, int BAND>
+__device__ __forceinline__ bool warp_band_solve(C (&W)[BAND + 1], C br, C *band, int N, int bw, C &xr) {
     constexpr unsigned kFull = 0xffffffffu;
-    const int r = threadIdx.x & 31, bw1 = bw + 1;
-    C Lr[kRegBand + 1];
-#pragma unroll
-    for (int d = 0; d <= kRegBand; ++d) Lr[d] = (r < N && d <= bw && d <= r) ? band[(size_t)r * bw1 + d] : C(0);
+    const int r = threadIdx.x & 31;
+    C acc = C(0), y = C(0), dinv = C(0);
+    bool ok = true;
+#pragma unroll 1
     for (int k = 0; k < N; ++k) {
-        const C piv = __shfl_sync(kFull, Lr[0], k);
-        if (!(piv > C(0))) return false;
+        const C piv = __shfl_sync(kFull, W[0], k);
+        ok = ok && piv > C(0);
         const C rkk = rsqrt_of<C>(piv);
-        if (r == k) Lr[0] = rkk;
-        const int dk = r - k;
-        C lk = C(0);   // L(r, k) once column k is scaled
+        const bool in = r > k && r <= k + bw && r < N;
+        const C lk = in ? W[0] * rkk : C(0);   // L(r, k)
+        C lc[BAND + 1];
 #pragma unroll
-        for (int d = 1; d <= kRegBand; ++d)
-            if (d == dk && d <= bw) {
-                Lr[d] *= rkk;
-                lk = Lr[d];
-            }
-        // trailing update: L(r, c) -= L(r, k) L(c, k) for k < c <= r <= k + bw
+        for (int j = 1; j <= BAND; ++j) lc[j] = __shfl_sync(kFull, lk, (k + j) & 31);
+        const C yk = __shfl_sync(kFull, (br - acc) * rkk, k);
+        dinv = r == k ? rkk : dinv;
+        y = r == k ? yk : y;
+        acc = in ? acc + lk * yk : acc;
+        if (in) band[k * bw + (r - k - 1)] = lk;
+        // trailing update: A(r, c) -= L(r, k) L(c, k) for k < c <= r <= k + bw, then the window slides
 #pragma unroll
-        for (int j = 1; j <= kRegBand; ++j) {
-            if (j > bw) break;
-            const C lck = __shfl_sync(kFull, lk, min(k + j, 31));
-            const int idx = dk - j;   // r - c
-#pragma unroll
-            for (int d = 0; d < kRegBand; ++d)
-                if (d == idx && dk <= bw && r < N) Lr[d] -= lk * lck;
+        for (int j = 1; j <= BAND; ++j) {
+            const C v = W[j] - lk * lc[j];
+            W[j] = in && k + j <= r ? v : W[j];
         }
-    }
-    // forward: y = L^-1 b
-    const C br = r < N ? b[r] : C(0);
-    C acc = C(0), y = C(0);
-    for (int c = 0; c < N; ++c) {
-        const C yc = __shfl_sync(kFull, (br - acc) * Lr[0], c);
-        if (r == c) y = yc;
-        const int dc = r - c;
 #pragma unroll
-        for (int d = 1; d <= kRegBand; ++d)
-            if (d == dc && d <= bw) acc += Lr[d] * yc;
+        for (int j = 0; j < BAND; ++j) W[j] = in ? W[j + 1] : W[j];
     }
-    // backward: x = L^-T y
-    C acc2 = C(0);
+    __syncwarp();
+    // backward: x = L^-T y; the column's entry of the next step is loaded ahead of the chain
+    auto entry = [&](int c) { return r < c && r >= c - bw ? band[r * bw + (c - r - 1)] : C(0); };   // L(c, r)
+    C acc2 = C(0), lcr = entry(N - 1);
     xr = C(0);
+#pragma unroll 1
     for (int c = N - 1; c >= 0; --c) {
-        const C xc = __shfl_sync(kFull, (y - acc2) * Lr[0], c);
-        if (r == c) xr = xc;
-#pragma unroll
-        for (int d = 1; d <= kRegBand; ++d) {
-            if (d > bw) break;
-            const C lcd = __shfl_sync(kFull, Lr[d], c);   // L(c, c - d)
-            if (r == c - d) acc2 += lcd * xc;
-        }
+        const C nxt = entry(c - 1);
+        const C xc = __shfl_sync(kFull, (y - acc2) * dinv, c);
+        xr = r == c ? xc : xr;
+        acc2 = r < c && r >= c - bw ? acc2 + lcr * xc : acc2;
+        lcr = nxt;
     }
-    return true;
+    return ok;
+}
+
+// The Picard iteration of coarse_solve_team for the tiny coarsest grids (N <= 32 cells, band
+// <= BAND), by one warp with one cell per lane (row-major) and everything in registers: the
+// neighbours' values come by shuffles, and the coefficients at an iterate serve both its residual
+// norm and the next system.  The operations, their order and the stopping tests are the general
+// routine's (FP32: the tests compare the squares of the norms, which decide the same way without
+// FP64 square roots).  On a 4 x 4 grid the two iterations of a V-cycle's solve took 42,000 cycles
+// in the general routine, a tenth of the bottom of the V-cycle.
+template <typename T, typename C, int BAND>
+__device__ __forceinline__ void coarse_solve_lanes(const CoarseGrid<T> &L, const ModelParams &mp, double A1frac,
+                                                double h2nm, int maxit, double tol, C *scratch, int *s_err,
+                                                int *it_out, double *res_out) {
+    constexpr unsigned kFull = 0xffffffffu;
+    using TM = Team<32>;
+    constexpr bool kF32 = sizeof(C) == 4;
+    constexpr C kStat = kF32 ? C(1e-6) : C(1e-14);
+    const int n = L.n, m = L.m, p = L.pitch, N = n * m;
+    const int q = threadIdx.x & 31;
+    const bool colmajor = m > n, own = q < N;
+    const int bw = colmajor ? n : m;
+    const C hinv = C(2) * (C)L.inv_2h;
+    const C cdiff = C(mp.mu) * hinv * hinv;
+    const C inv_tau = (C)L.inv_tau, inv_2h = (C)L.inv_2h, beta = (C)L.beta;
+    const int i = own ? q / m : 0, j = own ? q - i * m : 0;
+    const bool hS = own && i + 1 < n, hN = own && i > 0, hE = own && j + 1 < m, hW = own && j > 0;
+    const int qS = hS ? q + m : q, qN = hN ? q - m : q, qE = hE ? q + 1 : q, qW = hW ? q - 1 : q;
+    // cell (i, j) is row `row` of the system; lane q solves row q, which is cell `cell`
+    const int row = own ? (colmajor ? j * n + i : q) : q;
+    const int cell = own && colmajor ? (q - (q / n) * n) * m + q / n : q;
+    const int o = i * p + j;
+    const C pc = own ? (C)L.pn[o] : C(0);
+    const C pS = __shfl_sync(kFull, pc, qS), pN = __shfl_sync(kFull, pc, qN), pE = __shfl_sync(kFull, pc, qE),
+            pW = __shfl_sync(kFull, pc, qW);
+    const C w = L.wb ? C(__bfloat162float(L.wb[o])) : (C)L.w[o];
+    const C F = (C)L.F[o], rhs = L.has_rhs ? (C)L.rhs[o] : C(0);
+    C x = own ? (C)L.u[o] : C(0);
+    if (q == 0) *s_err = 0;
+    double r0 = 0.0, res = 0.0, res_prev = 0.0;   // residual norms (FP32: their squares)
+    int it = 0;
+#pragma unroll 1
+    for (;;) {
+        // G at phi = pn + x and the Rada-Chen area term
+        const C xS = __shfl_sync(kFull, x, qS), xN = __shfl_sync(kFull, x, qN), xE = __shfl_sync(kFull, x, qE),
+                xW = __shfl_sync(kFull, x, qW);
+        C area = C(0);
+        if (mp.model == 1) {
+            double hs = 0.0;
+            if (own) hs += 0.5 + atan(((double)pc + (double)x) / mp.eps) / M_PI;
+            hs = TM::template sum<double>(hs, nullptr);
+            area = (C)(2.0 * mp.nu * (h2nm * hs - A1frac));
+        }
+        const C gy = ((pS - pN) + (xS - xN)) * inv_2h;
+        const C gx = ((pE - pW) + (xE - xW)) * inv_2h;
+        const C g = w * rsqrt_of<C>(gx * gx + gy * gy + beta);
+        const C fS = C(0.5) * (g + __shfl_sync(kFull, g, qS)), fN = C(0.5) * (g + __shfl_sync(kFull, g, qN));
+        const C fE = C(0.5) * (g + __shfl_sync(kFull, g, qE)), fW = C(0.5) * (g + __shfl_sync(kFull, g, qW));
+        // the residual norm, and the row of the system (neighbours outside the grid add nothing)
+        C fl = C(0), diag = C(0), pflux = C(0);
+        auto add = [&](bool has, C f, C p2, C x2) {
+            const C a = cdiff * f;
+            const C fl2 = fl + f * ((p2 - pc) + (x2 - x)), dg2 = diag + a, pf2 = pflux + f * (p2 - pc);
+            fl = has ? fl2 : fl;
+            diag = has ? dg2 : diag;
+            pflux = has ? pf2 : pflux;
+            return has ? -a : C(0);
+        };
+        const C aS = add(hS, fS, pS, xS), aN = add(hN, fN, pN, xN), aE = add(hE, fE, pE, xE), aW = add(hW, fW, pW, xW);
+        (void)aS;
+        (void)aE;
+        const C Lv = cdiff * fl - F - area - inv_tau * x;
+        const C rr = rhs - Lv;
+        const C ss = TM::template sum<C>(own ? rr * rr : C(0), nullptr);
+        res = kF32 ? (double)ss : sqrt((double)ss);
+        if (it == 0) {
+            r0 = res;
+        } else {
+            if (res <= (kF32 ? tol * tol : tol) * r0 || res == 0.0) break;
+            if (kF32 && res > 0.81 * res_prev) break;
+        }
+        res_prev = res;
+        if (r0 == 0.0) break;
+        // row q of the system: the entries left of the diagonal are at distance 1 and bw
+        const C near_ = colmajor ? aN : aW, far_ = colmajor ? aW : aN;
+        const C rdiag = __shfl_sync(kFull, diag + inv_tau, cell), rnear = __shfl_sync(kFull, near_, cell),
+                rfar = __shfl_sync(kFull, far_, cell);
+        const C rb = __shfl_sync(kFull, cdiff * pflux - F - area - rhs, cell);
+        C W[BAND + 1];
+        const int base = max(q - bw, 0);
+#pragma unroll
+        for (int t = 0; t <= BAND; ++t) {
+            C v = C(0);
+            if (bw > 1 && base + t == q - 1) v = rnear;
+            if (q >= bw && t == 0) v = rfar;
+            if (base + t == q) v = rdiag;
+            W[t] = own ? v : C(0);
+        }
+        C xr;
+        if (!warp_band_solve<C, BAND>(W, own ? rb : C(0), scratch, N, bw, xr)) {
+            if (q == 0) *s_err = 1;
+            TM::sync();
+            break;
+        }
+        const C nx = __shfl_sync(kFull, xr, row);
+        C dmax = own ? max_t<C>(C(0), abs_t<C>(nx - x)) : C(0), pmax = own ? max_t<C>(C(1), abs_t<C>(pc + nx)) : C(1);
+        dmax = TM::template max<C>(dmax, nullptr);
+        pmax = TM::template max<C>(pmax, nullptr);
+        x = own ? nx : C(0);
+        ++it;
+        if (dmax <= kStat * pmax || it >= maxit) break;
+    }
+    if (own) stc(L.u, (size_t)o, (size_t)n * p, kDbgCoarse, (T)x);
+    *it_out = it;
+    *res_out = kF32 ? sqrt(res) : res;
+    TM::sync();
+}
+
+// coarse_solve_lanes where it is called: FP32 inline, FP64 as a function of its own, whose registers
+// (two a value) then do not crowd the calling kernel's.
+template <typename T, typename C, int BAND>
+__device__ __noinline__ void coarse_solve_lanes_call(const CoarseGrid<T> &L, const ModelParams &mp, double A1frac,
+                                                     double h2nm, int maxit, double tol, C *scratch, int *s_err,
+                                                     int *it_out, double *res_out) {
+    coarse_solve_lanes<T, C, BAND>(L, mp, A1frac, h2nm, maxit, tol, scratch, s_err, it_out, res_out);
+}
+template <typename T, typename C, int BAND>
+__device__ __forceinline__ void coarse_solve_tiny(const CoarseGrid<T> &L, const ModelParams &mp, double A1frac,
+                                                  double h2nm, int maxit, double tol, C *scratch, int *s_err,
+                                                  int *it_out, double *res_out) {
+    if (sizeof(C) == 4)
+        coarse_solve_lanes<T, C, BAND>(L, mp, A1frac, h2nm, maxit, tol, scratch, s_err, it_out, res_out);
+    else
+        coarse_solve_lanes_call<T, C, BAND>(L, mp, A1frac, h2nm, maxit, tol, scratch, s_err, it_out, res_out);
 }
 
 // Run by the NT threads of a team (NT = 32: warp 0; else the whole block) in the arithmetic
 // type C (storage T); scratch holds coarse_scratch_elems(n, m) values of C.
 template <typename T, typename C, int NT>
-__device__ void coarse_solve_team(const CoarseGrid<T> &L, ModelParams mp, double A1frac, double h2nm,
+__device__ __noinline__ void coarse_solve_team(const CoarseGrid<T> &L, ModelParams mp, double A1frac, double h2nm,
                                   int maxit, double tol, C *scratch, double *red, int *s_err,
                                   int *it_out, double *res_out) {
     using TM = Team<NT>;
@@ -238,66 +362,51 @@ __device__ void coarse_solve_team(const CoarseGrid<T> &L, ModelParams mp, double
             b[r] = cdiff * pflux - (C)L.F[o] - area - (L.has_rhs ? (C)L.rhs[o] : C(0));
         }
         TM::sync();
-        bool in_regs = false;
-        if constexpr (NT == 32) in_regs = N <= 32 && bw <= kRegBand;
-        if (in_regs) {
-            // the tiny coarsest grids: the band factor in registers, one row per lane
-            C xr;
-            const bool ok = warp_band_solve<C>(band, b, N, bw, xr);
+        // right-looking banded Cholesky: band[r*bw1 + (r-c)] = L(r, c); the diagonal entry
+        // keeps 1 / L(k, k) once column k is done
+        for (int k = 0; k < N && !(*s_err); ++k) {
+            if (tid == 0) {
+                C d = band[(size_t)k * bw1];
+                if (!(d > C(0))) (*s_err) = 1;
+                else band[(size_t)k * bw1] = rsqrt_of<C>(d);
+            }
             TM::sync();
-            if (!ok) {
-                if (tid == 0) *s_err = 1;
-                TM::sync();
-                break;
-            }
-            if (tid < N) b[tid] = xr;
-        } else {
-            // right-looking banded Cholesky: band[r*bw1 + (r-c)] = L(r, c); the diagonal entry
-            // keeps 1 / L(k, k) once column k is done
-            for (int k = 0; k < N && !(*s_err); ++k) {
-                if (tid == 0) {
-                    C d = band[(size_t)k * bw1];
-                    if (!(d > C(0))) (*s_err) = 1;
-                    else band[(size_t)k * bw1] = rsqrt_of<C>(d);
-                }
-                TM::sync();
-                if ((*s_err)) break;
-                const C rkk = band[(size_t)k * bw1];
-                const int last = min(k + bw, N - 1), cnt = last - k;
-                for (int t = tid; t < cnt; t += nt)
-                    if (MG_DBG_OK((size_t)(k + 1 + t) * bw1 + (1 + t), (size_t)N * bw1, kDbgCoarse))
-                        band[(size_t)(k + 1 + t) * bw1 + (1 + t)] *= rkk;
-                TM::sync();
-                for (int t = tid; t < cnt * cnt; t += nt) {
-                    // the trailing triangle: rows ii >= columns jj (integer indexing only)
-                    const int ii = t / cnt, jj = t - ii * cnt;
-                    if (jj > ii) continue;
-                    int ri = k + 1 + ii, rj = k + 1 + jj;
-                    if (!MG_DBG_OK((size_t)ri * bw1 + (ri - rj), (size_t)N * bw1, kDbgCoarse) ||
-                        !MG_DBG_OK(ri - k, bw1, kDbgCoarse) || !MG_DBG_OK(rj - k, bw1, kDbgCoarse))
-                        continue;
-                    band[(size_t)ri * bw1 + (ri - rj)] -= band[(size_t)ri * bw1 + (ri - k)] * band[(size_t)rj * bw1 + (rj - k)];
-                }
-                TM::sync();
-            }
             if ((*s_err)) break;
-            // forward and backward substitution by warp 0
-            if (tid < 32) {
-                for (int r = 0; r < N; ++r) {
-                    C s = C(0);
-                    for (int c = max(0, r - bw) + tid; c < r; c += 32) s += band[(size_t)r * bw1 + (r - c)] * y[c];
-                    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-                    if (tid == 0) y[r] = (b[r] - s) * band[(size_t)r * bw1];
-                    __syncwarp();
-                }
-                for (int r = N - 1; r >= 0; --r) {
-                    C s = C(0);
-                    int c1 = min(N - 1, r + bw);
-                    for (int c = r + 1 + tid; c <= c1; c += 32) s += band[(size_t)c * bw1 + (c - r)] * b[c];
-                    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-                    if (tid == 0) b[r] = (y[r] - s) * band[(size_t)r * bw1];
-                    __syncwarp();
-                }
+            const C rkk = band[(size_t)k * bw1];
+            const int last = min(k + bw, N - 1), cnt = last - k;
+            for (int t = tid; t < cnt; t += nt)
+                if (MG_DBG_OK((size_t)(k + 1 + t) * bw1 + (1 + t), (size_t)N * bw1, kDbgCoarse))
+                    band[(size_t)(k + 1 + t) * bw1 + (1 + t)] *= rkk;
+            TM::sync();
+            for (int t = tid; t < cnt * cnt; t += nt) {
+                // the trailing triangle: rows ii >= columns jj (integer indexing only)
+                const int ii = t / cnt, jj = t - ii * cnt;
+                if (jj > ii) continue;
+                int ri = k + 1 + ii, rj = k + 1 + jj;
+                if (!MG_DBG_OK((size_t)ri * bw1 + (ri - rj), (size_t)N * bw1, kDbgCoarse) ||
+                    !MG_DBG_OK(ri - k, bw1, kDbgCoarse) || !MG_DBG_OK(rj - k, bw1, kDbgCoarse))
+                    continue;
+                band[(size_t)ri * bw1 + (ri - rj)] -= band[(size_t)ri * bw1 + (ri - k)] * band[(size_t)rj * bw1 + (rj - k)];
+            }
+            TM::sync();
+        }
+        if ((*s_err)) break;
+        // forward and backward substitution by warp 0
+        if (tid < 32) {
+            for (int r = 0; r < N; ++r) {
+                C s = C(0);
+                for (int c = max(0, r - bw) + tid; c < r; c += 32) s += band[(size_t)r * bw1 + (r - c)] * y[c];
+                for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+                if (tid == 0) y[r] = (b[r] - s) * band[(size_t)r * bw1];
+                __syncwarp();
+            }
+            for (int r = N - 1; r >= 0; --r) {
+                C s = C(0);
+                int c1 = min(N - 1, r + bw);
+                for (int c = r + 1 + tid; c <= c1; c += 32) s += band[(size_t)c * bw1 + (c - r)] * b[c];
+                for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+                if (tid == 0) b[r] = (y[r] - s) * band[(size_t)r * bw1];
+                __syncwarp();
             }
         }
         TM::sync();
@@ -333,7 +442,7 @@ __device__ void coarse_solve_team(const CoarseGrid<T> &L, ModelParams mp, double
 // total-phi form, rewritten for phi = pn + u).  Scratch: 5 N values of C.
 // ---------------------------------------------------------------------------------------
 template <typename T, typename C, int NT>
-__device__ void aos_solve_team(const CoarseGrid<T> &L, ModelParams mp, double A1frac, double h2nm, int iters,
+__device__ __noinline__ void aos_solve_team(const CoarseGrid<T> &L, ModelParams mp, double A1frac, double h2nm, int iters,
                                double dt_, C *scratch, double *red) {
     using TM = Team<NT>;
     const int n = L.n, m = L.m, p = L.pitch, N = n * m;
@@ -429,7 +538,15 @@ __device__ void coarse_solve_block(const CoarseGrid<T> &L, ModelParams mp, doubl
         *res_out = 0.0;
         return;
     }
-    if (L.n * L.m <= kWarpCoarseMax) {
+    if (L.n * L.m <= 32) {   // the shorter side is then at most 5 cells
+        if (threadIdx.x < 32) {
+            if (min(L.n, L.m) <= 4)
+                coarse_solve_tiny<T, C, 4>(L, mp, A1frac, h2nm, maxit, tol, scratch, s_err, it_out, res_out);
+            else
+                coarse_solve_tiny<T, C, 5>(L, mp, A1frac, h2nm, maxit, tol, scratch, s_err, it_out, res_out);
+        }
+        __syncthreads();
+    } else if (L.n * L.m <= kWarpCoarseMax) {
         if (threadIdx.x < 32)
             coarse_solve_team<T, C, 32>(L, mp, A1frac, h2nm, maxit, tol, scratch, red, s_err, it_out, res_out);
         __syncthreads();
