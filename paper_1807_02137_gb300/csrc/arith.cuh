@@ -30,6 +30,14 @@ __device__ __forceinline__ double sqrt_rn(double a) { return __dsqrt_rn(a); }
 __device__ __forceinline__ float div_relax(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double div_relax(double a, double b) { return __ddiv_rn(a, b); }
 
+// The quotient a / b from r = recip_relax(b): in FP32 the approximate quotient is a times the
+// approximate reciprocal, so this is div_relax(a, b) to the bit and the reciprocal can be formed
+// once, ahead of its use; in FP64 (IEEE division) r is b itself.
+__device__ __forceinline__ float recip_relax(float b) { return __fdividef(1.0f, b); }
+__device__ __forceinline__ double recip_relax(double b) { return b; }
+__device__ __forceinline__ float div_by(float a, float r) { return __fmul_rn(a, r); }
+__device__ __forceinline__ double div_by(double a, double r) { return __ddiv_rn(a, r); }
+
 // Face coefficient of a face that exists: the arithmetic mean of the two cell values of
 // G = w / |grad phi|_beta (Sec. 2.2, eq. abcdrc: G_{i+1/2,j}); a boundary face carries no flux.
 template <typename T>
@@ -93,14 +101,63 @@ struct RunCell {
     T f;
 };
 
+// Parallel cyclic reduction of the tridiagonal rows a x(t-1) + b x(t) + c x(t+1) = d held one per
+// lane, whose couplings stay inside the runs of member cells mk (an identity row elsewhere): each
+// doubling step s = 1, 2, 4, 8, 16 eliminates the couplings to positions t - s and t + s.  Step s
+// is needed while some run is longer than s, which the mask alone tells: the vote on the next step
+// is under way during the current one, off the chain of shuffles.  A lane whose partner t -+ s
+// lies outside the piece has coupling 0 there and receives its own row from the shuffle: the step
+// adds 0 times finite values.
+template <typename T>
+__device__ __forceinline__ T pcr_rows(uint32_t mk, T a, T b, T c, T d) {
+    constexpr unsigned kFull = 0xffffffffu;
+    uint32_t run = mk & (mk >> 1);   // bit t: positions t .. t + s are members, s the step about to run
+    bool go = __any_sync(kFull, run != 0u);
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+        if (!go) break;
+        run &= run >> s;
+        go = __any_sync(kFull, run != 0u);
+        const T rb = recip_relax(b);
+        const T am = __shfl_up_sync(kFull, a, s), rm = __shfl_up_sync(kFull, rb, s);
+        const T cm = __shfl_up_sync(kFull, c, s), dm = __shfl_up_sync(kFull, d, s);
+        const T ap = __shfl_down_sync(kFull, a, s), rp = __shfl_down_sync(kFull, rb, s);
+        const T cp = __shfl_down_sync(kFull, c, s), dp = __shfl_down_sync(kFull, d, s);
+        const T al = div_by(-a, rm), ga = div_by(-c, rp);
+        b = fma_rn(ga, ap, fma_rn(al, cm, b));
+        d = fma_rn(ga, dp, fma_rn(al, dm, d));
+        a = mul_rn(al, am);
+        c = mul_rn(ga, cp);
+    }
+    return div_relax(d, b);
+}
+
+// This lane's row of a partial-line system: cell values ap, an (faces along the line), ax1, ax2
+// (across), nb = -(the diagonal), the values across and the line neighbours' values, which enter
+// the right-hand side where the neighbour is not a member.
+template <typename T>
+__device__ __forceinline__ T pcr_cell(uint32_t mk, int len, T cdiff, T ap, T an, T ax1, T ax2, T diag, T ux1, T ux2, T f,
+                                      T prevv, T nextv) {
+    const int lane = threadIdx.x & 31;
+    T a = T(0), b = T(1), c = T(0), d = T(0);
+    if ((mk >> lane) & 1u) {
+        const T lo = mul_rn(cdiff, ap), up = mul_rn(cdiff, an);
+        b = -diag;
+        const T across = fma_rn(ax2, ux2, mul_rn(ax1, ux1));
+        d = fma_rn(-cdiff, across, f);
+        const bool pm = lane > 0 && ((mk >> (lane - 1)) & 1u);
+        const bool nm = lane < 31 && lane + 1 < len && ((mk >> (lane + 1)) & 1u);
+        if (pm) a = lo; else d = fma_rn(-lo, prevv, d);
+        if (nm) c = up; else d = fma_rn(-up, nextv, d);
+    }
+    return pcr_rows<T>(mk, a, b, c, d);
+}
+
 // Partial-line update (Sec. 4.3, step III) of one 32-cell piece of a line, by a whole warp
 // (lane t: piece position t).  Each run of member cells (bit t of mk) is a tridiagonal system
 // coupled through the in-line coefficients, with the values just outside the run fixed; the
 // system is diagonally dominant (Sec. 3.2).  Every other lane carries an identity row, so the
-// runs decouple and one parallel cyclic reduction solves all of them at once: each doubling
-// step s = 1, 2, 4, 8, 16 eliminates the couplings to positions t - s and t + s, and the loop
-// stops as soon as no coupling is left (after ceil(log2(longest run)) steps; the remaining
-// steps would change no value).
+// runs decouple and one parallel cyclic reduction (pcr_rows) solves all of them at once.
 //   own         this lane's value at the start of the phase (0 for lanes >= len);
 //   endp, endn  the values just before / after the piece (their coefficients are zero at a
 //               domain edge);  at(t) the RunCell of position t (called for member lanes only).
@@ -115,35 +172,14 @@ __device__ __forceinline__ bool pcr_piece(uint32_t mk, int len, T cdiff, T inv_t
     T prevv = __shfl_up_sync(kFull, own, 1), nextv = __shfl_down_sync(kFull, own, 1);
     if (lane == 0) prevv = endp;
     if (lane == len - 1) nextv = endn;
-    T a = T(0), b = T(1), c = T(0), d = T(0);
+    RunCell<T> cc{};
+    T diag = T(1);
     if (mem) {
-        const RunCell<T> cc = at(lane);
-        const T lo = mul_rn(cdiff, cc.ap), up = mul_rn(cdiff, cc.an);
+        cc = at(lane);
         const T sum = add_rn(add_rn(cc.ap, cc.an), add_rn(cc.ax1, cc.ax2));
-        b = -fma_rn(cdiff, sum, inv_tau);
-        const T across = fma_rn(cc.ax2, cc.ux2, mul_rn(cc.ax1, cc.ux1));
-        d = fma_rn(-cdiff, across, cc.f);
-        const bool pm = lane > 0 && ((mk >> (lane - 1)) & 1u);
-        const bool nm = lane < 31 && lane + 1 < len && ((mk >> (lane + 1)) & 1u);
-        if (pm) a = lo; else d = fma_rn(-lo, prevv, d);
-        if (nm) c = up; else d = fma_rn(-up, nextv, d);
+        diag = fma_rn(cdiff, sum, inv_tau);
     }
-#pragma unroll
-    for (int s = 1; s < 32; s <<= 1) {
-        if (!__any_sync(kFull, a != T(0) || c != T(0))) break;
-        T am = __shfl_up_sync(kFull, a, s), bm = __shfl_up_sync(kFull, b, s);
-        T cm = __shfl_up_sync(kFull, c, s), dm = __shfl_up_sync(kFull, d, s);
-        T ap = __shfl_down_sync(kFull, a, s), bp = __shfl_down_sync(kFull, b, s);
-        T cp = __shfl_down_sync(kFull, c, s), dp = __shfl_down_sync(kFull, d, s);
-        if (lane < s) { am = T(0); bm = T(1); cm = T(0); dm = T(0); }
-        if (lane + s > 31) { ap = T(0); bp = T(1); cp = T(0); dp = T(0); }
-        const T al = div_relax(-a, bm), ga = div_relax(-c, bp);
-        b = fma_rn(ga, ap, fma_rn(al, cm, b));
-        d = fma_rn(ga, dp, fma_rn(al, dm, d));
-        a = mul_rn(al, am);
-        c = mul_rn(ga, cp);
-    }
-    x = div_relax(d, b);
+    x = pcr_cell<T>(mk, len, cdiff, cc.ap, cc.an, cc.ax1, cc.ax2, diag, cc.ux1, cc.ux2, cc.f, prevv, nextv);
     return mem;
 }
 

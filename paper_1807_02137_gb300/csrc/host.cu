@@ -271,6 +271,7 @@ struct Solver final : SolverBase {
     int learn_skip = 0, learn_backoff = 1;   // plain V-cycles left before the next learned try
     long long learned_acc = 0, learned_rej = 0;
     size_t lb_smem = 0;
+    int lb_pad = 0, lc_pad = 0;   // odd row pitches in the bottom kernels' shared memory
     ModelParams mp{};
 
     ~Solver() override { release(); }
@@ -419,11 +420,21 @@ struct Solver final : SolverBase {
         if (tiles > kClusterMaxTiles) return;
         int ns[kMaxLevels], ms[kMaxLevels];
         for (int k = 0; k < nlev; ++k) { ns[k] = lv[k].n; ms[k] = lv[k].m; }
-        const size_t bytes = cluster_smem_bytes(bottom_smem_bytes(ns, ms, l + 1, nlev, p.precision == MG_MIXED));
-        if (cluster_fits(tiles, bytes) < 1) return;
+        if (fit_cluster(l, tiles, ns, ms) < 1) return;
         lc = l;   // the one-block kernel's start (lb) stays: it takes over if the cluster is switched off
         lc_tiles = tiles;
-        lc_smem = bytes;
+    }
+
+    // Shared memory of the cluster kernel from grid l (lc_smem, lc_pad: with odd row pitches if those
+    // fit, else dense); returns how many such clusters fit (see cluster_fits).
+    int fit_cluster(int l, int tiles, const int *ns, const int *ms) {
+        int fits = 0;
+        for (int pad = 1; pad >= 0; --pad) {
+            lc_pad = pad;
+            lc_smem = cluster_smem_bytes(bottom_smem_bytes(ns, ms, l + 1, nlev, p.precision == MG_MIXED, pad));
+            if ((fits = cluster_fits(tiles, lc_smem)) >= 1) return fits;
+        }
+        return fits;
     }
 
     // The bottom kernel runs grids lb .. nlev-1 in one block when the storage is FP32 (or mixed),
@@ -439,7 +450,7 @@ struct Solver final : SolverBase {
             int ns[kMaxLevels], ms[kMaxLevels];
             for (int l = 0; l < nlev; ++l) { ns[l] = lv[l].n; ms[l] = lv[l].m; }
             for (int l = nlev - 2; l >= 0; --l) {
-                size_t b = bottom_smem_bytes(ns, ms, l, nlev, p.precision == MG_MIXED);
+                size_t b = bottom_smem_bytes(ns, ms, l, nlev, p.precision == MG_MIXED, 0);
                 if (b > kBottomSmemMax) break;
                 lb_first = l;
             }
@@ -457,7 +468,12 @@ struct Solver final : SolverBase {
         int ns[kMaxLevels], ms[kMaxLevels];
         for (int k = 0; k < nlev; ++k) { ns[k] = lv[k].n; ms[k] = lv[k].m; }
         lb = l;
-        lb_smem = l >= 0 ? bottom_smem_bytes(ns, ms, l, nlev, p.precision == MG_MIXED) : 0;
+        lb_pad = 0;
+        lb_smem = 0;
+        if (l < 0) return;
+        lb_smem = bottom_smem_bytes(ns, ms, l, nlev, p.precision == MG_MIXED, 1);
+        lb_pad = lb_smem <= kBottomSmemPad;
+        if (!lb_pad) lb_smem = bottom_smem_bytes(ns, ms, l, nlev, p.precision == MG_MIXED, 0);
     }
 
     // The cluster bottom kernel from grid `level`: grids level+1 .. nlev-1 must fit the one-block
@@ -474,15 +490,13 @@ struct Solver final : SolverBase {
         int ns[kMaxLevels], ms[kMaxLevels];
         for (int k = 0; k < nlev; ++k) { ns[k] = lv[k].n; ms[k] = lv[k].m; }
         const int tiles = ((lv[level].n + 31) / 32) * ((lv[level].m + 31) / 32);
-        const size_t bytes = cluster_smem_bytes(bottom_smem_bytes(ns, ms, level + 1, nlev, p.precision == MG_MIXED));
-        const int fits = cluster_fits(tiles, bytes);
+        const int fits = fit_cluster(level, tiles, ns, ms);
         if (fits < 1)
             return fail(MG_ERR_ARG, "the grid does not fit one thread-block cluster (" + std::to_string(tiles) +
-                                        " CTAs, " + std::to_string(bytes) + " bytes of shared memory each: " +
+                                        " CTAs, " + std::to_string(lc_smem) + " bytes of shared memory each: " +
                                         std::to_string(fits) + ")");
         lc = level;
         lc_tiles = tiles;
-        lc_smem = bytes;
         drop_graphs();
         return MG_OK;
     }
@@ -540,9 +554,11 @@ struct Solver final : SolverBase {
             BottomArgs a{};
             a.lb = first; a.L = nlev; a.nu1 = p.nu1; a.nu2 = p.nu2;
             a.coarse_fp64 = p.precision == MG_MIXED;
+            a.pad = cluster ? lc_pad : lb_pad;
             a.coarse_aos = p.coarse_solver == MG_COARSE_AOS;
             a.aos_dt = p.aos_dt;
             for (int l = first; l < nlev; ++l) a.g[l] = view(l);
+            a.first = a.g[first];
             a.mp = mp;
             a.A1frac = A1 / ((double)n * m);
             a.h2nm_coarse = h2nm(nlev - 1);

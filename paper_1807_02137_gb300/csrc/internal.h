@@ -282,16 +282,20 @@ struct BottomArgs {
     int lb, L, nu1, nu2;
     int coarse_fp64;   // the coarsest solve in FP64 arithmetic (mixed precision) or FP32
     int coarse_aos;    // the coarsest solve by AOS iterations (step aos_dt)
+    int pad;           // odd row pitches in shared memory (where they fit, see bottom_smem_bytes)
     double aos_dt;
+    LevelView<float> first;   // grid lb
     LevelView<float> g[kMaxLevels];
     ModelParams mp;
     double A1frac, h2nm_coarse, coarse_tol;
     int coarse_maxit;
     Scalars *sc;
 };
-constexpr size_t kBottomSmemMax = 200 * 1024;
+constexpr size_t kBottomSmemMax = 200 * 1024, kBottomSmemPad = 216 * 1024;
 constexpr int kBottomThreads = 1024;   // threads of the bottom kernels' blocks
-size_t bottom_smem_bytes(const int *n, const int *m, int lb, int L, int coarse_fp64);
+// Shared memory of grids lb .. L-1; pad: with odd row pitches.  Whether a first grid fits is decided
+// without the padding (kBottomSmemMax); the padding is used where it still fits kBottomSmemPad.
+size_t bottom_smem_bytes(const int *n, const int *m, int lb, int L, int coarse_fp64, int pad);
 void prepare_bottom_kernel();
 void launch_bottom(const BottomArgs &A, size_t smem, cudaStream_t st);
 // The bottom of the V-cycle from grid A.lb spread over a cluster of `tiles` CTAs (one per 32 x 32
@@ -299,7 +303,7 @@ void launch_bottom(const BottomArgs &A, size_t smem, cudaStream_t st);
 // of the shared memory of grids A.lb+1 .. L-1; cluster_fits returns how many such clusters can
 // be resident (0: none or out of range; negative: minus the CUDA error of the query).
 constexpr int kClusterMaxTiles = 16;
-constexpr size_t kClusterSmemMax = 220 * 1024;   // dynamic, beside the kernel's static shared memory
+constexpr size_t kClusterSmemMax = 222 * 1024;   // dynamic, beside the kernel's static shared memory
 size_t cluster_smem_bytes(size_t bottom_bytes);
 int cluster_fits(int tiles, size_t smem);
 void launch_cluster(const BottomArgs &A, int tiles, size_t smem, cudaStream_t st);
