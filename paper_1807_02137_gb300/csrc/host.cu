@@ -192,7 +192,7 @@ struct Level {
     uint32_t *mrow = nullptr, *mcol = nullptr;
     __nv_bfloat16 *wb = nullptr;   // mixed precision only
     uint8_t *cls = nullptr;        // Hybrid Smoother 1 only
-    SweepMaps maps[kTileShapes];   // FP32 storage: tensor maps of the TMA sweep, per tile shape
+    SweepMaps maps[kSweepMaps];    // FP32 storage: tensor maps of the TMA sweep, per tile shape
     SnapMaps smaps;                // FP32 storage: tensor maps of the TMA snapshot
     ResMaps rmaps;                 // FP32 storage: tensor maps of the TMA residual kernels
 };
@@ -386,7 +386,7 @@ struct Solver final : SolverBase {
         if constexpr (std::is_same<T, float>::value) {
             if (p.smoother == MG_SMOOTH_FUSED)
                 for (int l = 0; l < nlev; ++l)
-                    for (int sh = 0; sh < kTileShapes; ++sh)
+                    for (int sh = 0; sh < kSweepMaps; ++sh)
                         if (!encode_sweep_maps(view(l), sh, &lv[l].maps[sh]))
                             return fail(MG_ERR_CUDA, "cuTensorMapEncodeTiled failed for a grid");
             for (int l = 0; l < nlev; ++l)
@@ -756,7 +756,7 @@ struct Solver final : SolverBase {
             launch_sweep_fused<T>(v, k, sh, st);
         } else {
             if constexpr (std::is_same<T, float>::value)
-                launch_sweep_tma(v, k, sh, lv[l].maps[sh], &dsc->err, wait_limit, st);
+                launch_sweep_tma(v, k, sh, lv[l].maps, &dsc->err, wait_limit, st);
             else launch_sweep_fused<T>(v, k, sh, st);
         }
     }

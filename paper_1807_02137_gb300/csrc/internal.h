@@ -153,6 +153,9 @@ template <typename T>
 void launch_snapshot(const LevelView<T> &L, const double *area, cudaStream_t st);
 constexpr int kTileShapes = 6;   // fused-sweep tile shapes (rows x columns, threads): 32x64 256, 32x32 128,
                                  // 64x64 512, 32x64 512, 32x32 256, 32x32 512 (see smooth_kernels.cu)
+// further tensor maps of the TMA sweep: the thin tiles of row and of column sweeps, which shapes 4
+// and 5 (32x32) run as on small grids
+constexpr int kThinRows = kTileShapes, kThinCols = kTileShapes + 1, kSweepMaps = kTileShapes + 2;
 template <typename T>
 void launch_sweep_fused(const LevelView<T> &L, int sweep, int shape, cudaStream_t st);
 template <typename T>
@@ -235,7 +238,8 @@ bool encode_sweep_maps(const LevelView<float> &L, int shape, SweepMaps *M);
 // tensor map with box RW x RH (zero fill outside the grid); false when the driver refuses it.
 bool encode_map_2d(void *out, void *base, int elem, int n, int m, int pitch, int RH, int RW);
 constexpr long long kDefaultWaitLimit = 1LL << 22;   // try_wait rounds before a TMA wait gives up
-void launch_sweep_tma(const LevelView<float> &L, int sweep, int shape, const SweepMaps &M, int *err,
+// maps: the grid's kSweepMaps tensor-map sets, by shape.
+void launch_sweep_tma(const LevelView<float> &L, int sweep, int shape, const SweepMaps *maps, int *err,
                       long long wait_limit, cudaStream_t st);
 
 // learned.cu: learned relaxation weights (inference and training)

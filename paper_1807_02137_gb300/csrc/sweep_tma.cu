@@ -32,15 +32,18 @@ namespace {
 constexpr int kH = 4;
 constexpr long long kDrainLimit = 1LL << 22;   // try_wait rounds of the last wait for copies in flight
 
-template <int OH_, int OW_, int NT_, int MINB_ = 1, bool ONE_ = false>
+template <int OH_, int OW_, int NT_, int MINB_ = 1, bool ONE_ = false, int PW_ = OW_ + 2 * kH>
 struct TShape {
     static constexpr int OH = OH_, OW = OW_, NT = NT_;
+    static constexpr int PW = PW_;            // columns of the box in shared memory (its row pitch)
     static constexpr int MinBlocks = MINB_;   // resident blocks per SM asked of the compiler
     static constexpr bool OneTile = ONE_;     // always one tile per block (one stage), any grid size
     static constexpr int RH = OH + 2 * kH, RW = OW + 2 * kH;
     static constexpr int RowPieces = OW / 32 + 2, ColPieces = OH / 32 + 2;
     static constexpr int MkLines = RH > RW ? RH : RW, MkPieces = RowPieces > ColPieces ? RowPieces : ColPieces;
-    static constexpr int BoxBytes = RH * RW * 4;
+    static constexpr int BoxBytes = RH * PW * 4;
+    // pieces of 32 cells of a line in the tile (0 in a direction the shape does not serve)
+    static_assert(OW % 32 == 0 || OH % 32 == 0, "a tile holds whole line pieces in one direction at least");
 };
 // 6 blocks of 256 threads per SM (at most 42 registers), one tile and one stage per block: the
 // register limit, not shared memory, is what bounds the resident blocks, and six blocks each
@@ -58,11 +61,24 @@ using TT4 = TShape<32, 32, 256, 8>;
 // one block per SM and running persistent: 7.0 against 5.4 us per launch)
 using TT5 = TShape<32, 32, 512, 2>;
 
+// Thin tiles for grids that leave most SMs idle with 32 x 32 tiles (128^2: 16 of them): a quarter of
+// the rows (row sweeps A, B) or columns (column sweeps C, D) a block, so that four times the blocks
+// share the work.  A sweep of such a grid is one wave of blocks, and a block's time is its
+// instructions times its warps over the SM's four schedulers: the thin tile's checkerboard phase is
+// one cell a thread (320 cells of a colour in the box) and its line phases one line a warp.  The halo
+// costs more (1.9 computed cells per output cell against 1.3), which is why larger grids keep the
+// square tiles (see launch_thin).  Column tiles have rows of 20 floats: a column piece meets 4-way
+// bank conflicts with that pitch, 16-way with 16.
+using TTR = TShape<8, 32, 320, 4, true>;
+using TTC = TShape<32, 8, 320, 4, true, 20>;
+
 template <typename TS, int STAGES>
 struct TmaSmem {
-    float box[STAGES][3][TS::RH][TS::RW];      // [stage][u, G, f][row][column]
+    float box[STAGES][3][TS::RH][TS::PW];      // [stage][u, G, f][row][column]
     uint32_t mk[TS::MkLines][TS::MkPieces];    // member masks of the tile (as k_sweep)
     unsigned long long bar[STAGES];            // one mbarrier per stage
+    unsigned flags;                            // of the tile: 1 a solved piece has members, 2 a staged
+                                               // piece has, 4 a copy timed out
 };
 
 
@@ -78,11 +94,11 @@ __device__ __forceinline__ bool member(const TmaSmem<TS, STAGES> &S, int a, int 
 template <typename TS, int STAGES, int SWEEP, bool INTERIOR, bool WEIGHTED, bool MEMBERS = true>
 __device__ __forceinline__ void rb_phase(TmaSmem<TS, STAGES> &S, int st, const LevelView<float> &L, int ph, int i0,
                                          int j0) {
-    constexpr int kRH = TS::RH, kRW = TS::RW;
+    constexpr int kRH = TS::RH, kRW = TS::RW, kPW = TS::PW;
     constexpr bool rev = (SWEEP & 1) != 0;
-    float (*u)[kRW] = S.box[st][0];
-    const float (*G)[kRW] = S.box[st][1];
-    const float (*f)[kRW] = S.box[st][2];
+    float (*u)[kPW] = S.box[st][0];
+    const float (*G)[kPW] = S.box[st][1];
+    const float (*f)[kPW] = S.box[st][2];
     const int colour = rev ? 1 - ph : ph, lo = 1 + ph;
     const int n = L.n, m = L.m;
     const float c2 = L.cdiff * 0.5f;   // with face2 (see arith.cuh)
@@ -118,7 +134,7 @@ __global__ void __launch_bounds__(TS::NT, TS::MinBlocks) k_sweep_tma(LevelView<f
                                                       const __grid_constant__ CUtensorMap tG,
                                                       const __grid_constant__ CUtensorMap tf, int *err,
                                                       long long wait_limit) {
-    constexpr int kOH = TS::OH, kOW = TS::OW, kRH = TS::RH, kRW = TS::RW;
+    constexpr int kOH = TS::OH, kOW = TS::OW, kRH = TS::RH, kRW = TS::RW, kPW = TS::PW;
     constexpr int kRowPieces = TS::RowPieces, kColPieces = TS::ColPieces;
     constexpr bool rowwise = SWEEP < 2, rev = (SWEEP & 1) != 0;
     extern __shared__ unsigned char smem_raw[];
@@ -189,6 +205,7 @@ __global__ void __launch_bounds__(TS::NT, TS::MinBlocks) k_sweep_tma(LevelView<f
     uint32_t mw[kMaskPer];
     load_masks(tile, mw);
     if (tid == 0) {   // the thread that initialises the barriers issues the first tile's copies
+        S.flags = 0;
         for (int k = 0; k < STAGES; ++k) mbar_init(&S.bar[k], 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         if (tile < ntiles) issue(tile, 0);
@@ -205,7 +222,11 @@ __global__ void __launch_bounds__(TS::NT, TS::MinBlocks) k_sweep_tma(LevelView<f
         const bool lm = store_masks(mw, anym);
         load_masks(next, mw);   // in flight while this tile is smoothed (zeros past the last tile)
         const bool ok = mbar_wait(&S.bar[st], parity, wait_limit);
-        if (__syncthreads_or(!ok)) {
+        const unsigned fl = __reduce_or_sync(0xffffffffu, (lm ? 1u : 0u) | (anym ? 2u : 0u) | (ok ? 0u : 4u));
+        if ((tid & 31) == 0 && fl) atomicOr(&S.flags, fl);
+        __syncthreads();
+        const unsigned flags = S.flags;
+        if (flags & 4u) {
             // a copy did not complete within wait_limit rounds: report, give the copies in flight a
             // last bounded wait (kDrainLimit rounds, so that none still writes into shared memory
             // once the block has ended), stop
@@ -217,11 +238,11 @@ __global__ void __launch_bounds__(TS::NT, TS::MinBlocks) k_sweep_tma(LevelView<f
             __syncthreads();
             return;
         }
-        const bool lines = __syncthreads_or(lm);
-        const bool members = __syncthreads_or(anym);   // else the checkerboard skips no cell
-        float (*u)[kRW] = S.box[st][0];
-        const float (*G)[kRW] = S.box[st][1];
-        const float (*f)[kRW] = S.box[st][2];
+        const bool lines = flags & 1u;
+        const bool members = flags & 2u;   // else the checkerboard skips no cell
+        float (*u)[kPW] = S.box[st][0];
+        const float (*G)[kPW] = S.box[st][1];
+        const float (*f)[kPW] = S.box[st][2];
         // ---- checkerboard phases (distance 3 then 2 from the output tile)
         const bool interior = i0 - kH >= 0 && i0 - kH + kRH <= n && j0 - kH >= 0 && j0 - kH + kRW <= m;
 #pragma unroll
@@ -238,6 +259,7 @@ __global__ void __launch_bounds__(TS::NT, TS::MinBlocks) k_sweep_tma(LevelView<f
                 }
             }
             __syncthreads();
+            if (ph == 0 && tid == 0) S.flags = 0;   // for the next tile (every thread has read them)
         }
         // ---- partial-line phases (line_phase.cuh), skipped when no piece of the tile has a member
         if (lines)
@@ -283,7 +305,9 @@ void set_attr() {
 template <typename TS>
 void set_attrs() {
     set_attr<0, TS, 1>(); set_attr<1, TS, 1>(); set_attr<2, TS, 1>(); set_attr<3, TS, 1>();
-    set_attr<0, TS, 2>(); set_attr<1, TS, 2>(); set_attr<2, TS, 2>(); set_attr<3, TS, 2>();
+    if constexpr (!TS::OneTile) {
+        set_attr<0, TS, 2>(); set_attr<1, TS, 2>(); set_attr<2, TS, 2>(); set_attr<3, TS, 2>();
+    }
 }
 
 // One tile per block (one stage) when the shape asks for it or when every tile gets a resident
@@ -296,9 +320,26 @@ void launch_one(const LevelView<float> &L, const SweepMaps &M, int sms, int *err
     const CUtensorMap &mf = *reinterpret_cast<const CUtensorMap *>(M.f);
     if (TS::OneTile || ntiles <= sms * tma_blocks_per_sm<SW, TS, 1>()) {
         k_sweep_tma<SW, TS, 1><<<ntiles, TS::NT, tma_smem<SW, TS, 1>(), st>>>(L, *in, mG, mf, err, wl);
-    } else {
+    } else if constexpr (!TS::OneTile) {
         const int grid = std::min(ntiles, sms * tma_blocks_per_sm<SW, TS, 2>());
         k_sweep_tma<SW, TS, 2><<<grid, TS::NT, tma_smem<SW, TS, 2>(), st>>>(L, *in, mG, mf, err, wl);
+    }
+}
+
+// The thin tiles: on grids whose thin blocks are all resident at once.
+constexpr int kThinPerSm = 4;
+bool use_thin(const LevelView<float> &L, int sms) {
+    const long rows = (long)((L.m + 31) / 32) * ((L.n + 7) / 8), cols = (long)((L.m + 7) / 8) * ((L.n + 31) / 32);
+    return std::max(rows, cols) <= (long)sms * kThinPerSm;
+}
+
+void launch_thin(const LevelView<float> &L, int sweep, const SweepMaps &R, const SweepMaps &C, int sms, int *err,
+                 long long wl, cudaStream_t st) {
+    switch (sweep) {
+        case 0: launch_one<0, TTR>(L, R, sms, err, wl, st); break;
+        case 1: launch_one<1, TTR>(L, R, sms, err, wl, st); break;
+        case 2: launch_one<2, TTC>(L, C, sms, err, wl, st); break;
+        default: launch_one<3, TTC>(L, C, sms, err, wl, st); break;
     }
 }
 
@@ -337,8 +378,8 @@ bool encode(void *out, float *base, int n, int m, int pitch, int RH, int RW) {
 
 template <typename TS>
 bool encode_shape(const LevelView<float> &L, SweepMaps &M) {
-    return encode(M.u, L.u, L.n, L.m, L.pitch, TS::RH, TS::RW) && encode(M.t, L.t, L.n, L.m, L.pitch, TS::RH, TS::RW) &&
-           encode(M.G, L.G, L.n, L.m, L.pitch, TS::RH, TS::RW) && encode(M.f, L.f, L.n, L.m, L.pitch, TS::RH, TS::RW);
+    return encode(M.u, L.u, L.n, L.m, L.pitch, TS::RH, TS::PW) && encode(M.t, L.t, L.n, L.m, L.pitch, TS::RH, TS::PW) &&
+           encode(M.G, L.G, L.n, L.m, L.pitch, TS::RH, TS::PW) && encode(M.f, L.f, L.n, L.m, L.pitch, TS::RH, TS::PW);
 }
 
 int g_sms = 0;
@@ -362,6 +403,7 @@ bool encode_map_2d(void *out, void *base, int elem, int n, int m, int pitch, int
 
 void prepare_sweep_tma() {
     set_attrs<TT0>(); set_attrs<TT1>(); set_attrs<TT2>(); set_attrs<TT3>(); set_attrs<TT4>(); set_attrs<TT5>();
+    set_attr<0, TTR, 1>(); set_attr<1, TTR, 1>(); set_attr<2, TTC, 1>(); set_attr<3, TTC, 1>();
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
     if (g_sms < 1) g_sms = 1;
@@ -373,12 +415,19 @@ bool encode_sweep_maps(const LevelView<float> &L, int shape, SweepMaps *M) {
     if (shape == 3) return encode_shape<TT3>(L, *M);
     if (shape == 4) return encode_shape<TT4>(L, *M);
     if (shape == 5) return encode_shape<TT5>(L, *M);
+    if (shape == kThinRows) return encode_shape<TTR>(L, *M);
+    if (shape == kThinCols) return encode_shape<TTC>(L, *M);
     return encode_shape<TT0>(L, *M);
 }
 
-void launch_sweep_tma(const LevelView<float> &L, int sweep, int shape, const SweepMaps &M, int *err,
+void launch_sweep_tma(const LevelView<float> &L, int sweep, int shape, const SweepMaps *maps, int *err,
                       long long wait_limit, cudaStream_t st) {
     const long long wl = wait_limit;
+    const SweepMaps &M = maps[shape];
+    if (shape >= 4 && use_thin(L, g_sms)) {
+        launch_thin(L, sweep, maps[kThinRows], maps[kThinCols], g_sms, err, wl, st);
+        return;
+    }
     if (shape == 1) launch_shape<TT1>(L, sweep, M, g_sms, err, wl, st);
     else if (shape == 2) launch_shape<TT2>(L, sweep, M, g_sms, err, wl, st);
     else if (shape == 3) launch_shape<TT3>(L, sweep, M, g_sms, err, wl, st);
