@@ -14,6 +14,7 @@
 #include "arith.cuh"
 #include "coarse_body.cuh"
 #include "reduce.cuh"
+#include "tma.cuh"
 
 #include <algorithm>
 
@@ -446,7 +447,7 @@ __device__ __forceinline__ void tile_sync(int nt) {
     else asm volatile("bar.sync 1, %0;\n" ::"r"(nt) : "memory");
 }
 
-// One outer smoothing iteration: the snapshot and the four sweeps.  fas (not CL): the grid's first
+// One outer smoothing iteration: the snapshot and the four sweeps.  fas: the grid's first
 // snapshot after the restriction (u = u0) also completes the FAS right-hand side, rhs += L(pn + u0).
 // Not CL: run by the warps that own a row or a column of the grid (w < max(n, m)); the caller's
 // other warps wait at the block barrier after it.
@@ -493,7 +494,7 @@ __device__ __forceinline__ void tile_smooth(const TileArgs &A, TileScratch &S, C
         ds = fma_rn(aE, sub_rn(pE, pc), ds);
         ds = fma_rn(aW, sub_rn(pW, pc), ds);
         float base = add_rn(smf[A.F + oc], 0.0f);
-        if (!CL && fas) {   // as b_residual, mode 1, with uu = u (= u0 here)
+        if (fas) {   // as b_residual, mode 1, with uu = u (= u0 here)
             const float uc = U[o];
             float fl = mul_rn(aS, add_rn(sub_rn(pS, pc), sub_rn(U[oS], uc)));
             fl = fma_rn(aN, add_rn(sub_rn(pN, pc), sub_rn(U[oN], uc)), fl);
@@ -757,10 +758,22 @@ __device__ __forceinline__ void bottom_setup(const BottomArgs &A, BGrid *Bs, int
             smf[B.pn + q] = ldc(G.pn, o, lim, kDbgBottom);
             smf[B.w + q] = weight_at(G, o);
             smf[B.F + q] = ldc(G.F, o, lim, kDbgBottom);
-            if (load_first && l == lb) {
-                smf[B.u + q] = ldc(G.u, o, lim, kDbgBottom);
-                smf[B.rhs + q] = G.has_rhs ? ldc(G.rhs, o, lim, kDbgBottom) : 0.f;
-            }
+        }
+    }
+    pdl_wait();      // what lies above is fixed during a step; grid lb's u and rhs come from the
+    pdl_trigger();   // kernel before
+    if (load_first) {
+        const LevelView<float> &G = A.first;
+        const BGrid &B = Bs[lb];
+        const Map2 M = map_for(B.m);
+        FOR_CELLS(M, B.n, B.m, i, j) {
+            const int q = i * B.P + j;
+            const size_t o = (size_t)i * G.pitch + j, lim = (size_t)G.n * G.pitch;
+            if (!MG_DBG_OK(o, lim, kDbgBottom)) continue;
+            const float u = __ldcg(G.u + o);
+            smf[B.u + q] = u;
+            smf[B.u0 + q] = u;
+            smf[B.rhs + q] = G.has_rhs ? __ldcg(G.rhs + o) : 0.f;
         }
     }
     __syncthreads();
@@ -774,7 +787,7 @@ __global__ void __launch_bounds__(kBT) k_bottom(const __grid_constant__ BottomAr
     __shared__ TileScratch ts;
     unsigned char *sm = reinterpret_cast<unsigned char *>(smf);
     bottom_setup(A, Bs, A.lb, true, 0, s_off);
-    bottom_subcycle(A, Bs, A.lb, false, sm + s_off[0], reinterpret_cast<float *>(sm + s_off[1]), ts, sm + s_off[2], red,
+    bottom_subcycle(A, Bs, A.lb, A.fas != 0, sm + s_off[0], reinterpret_cast<float *>(sm + s_off[1]), ts, sm + s_off[2], red,
                     &s_err);
     // ---- grid lb's increment back to global memory
     {
@@ -838,15 +851,21 @@ __global__ void __launch_bounds__(kBT) k_cluster(const __grid_constant__ BottomA
         if (c.own) {
             const size_t o = (size_t)c.i * Lg.pitch + c.j, lim = (size_t)n * Lg.pitch;
             T.P[c.r0][c.c0] = ldc(Lg.pn, o, lim, kDbgBottom);
-            T.U[c.r0][c.c0] = ldc(Lg.u, o, lim, kDbgBottom);
             T.W[c.ti][c.lane] = weight_at(Lg, o);
             T.F[c.ti][c.lane] = ldc(Lg.F, o, lim, kDbgBottom);
-            T.R[c.ti][c.lane] = has_rhs ? ldc(Lg.rhs, o, lim, kDbgBottom) : 0.f;
         }
     }
     // grids lc+1 .. L-1: every CTA carves the same offsets (CTA 0's arrays are then reached by
     // mapping this CTA's addresses); their pn, w, F are loaded
-    bottom_setup(A, Bs, lc + 1, false, kTileBytes, s_off);
+    bottom_setup(A, Bs, lc + 1, false, kTileBytes, s_off);   // (waits for the kernel before)
+    {
+        const Cell c = cell_of_thread();
+        const size_t o = (size_t)c.i * Lg.pitch + c.j, lim = (size_t)n * Lg.pitch;
+        if (c.own && MG_DBG_OK(o, lim, kDbgBottom)) {
+            T.U[c.r0][c.c0] = __ldcg(Lg.u + o);
+            T.R[c.ti][c.lane] = has_rhs ? __ldcg(Lg.rhs + o) : 0.f;
+        }
+    }
     cluster_sync();   // every CTA of the cluster runs: its shared memory may be written
     {
         const Cell c = cell_of_thread();
@@ -864,7 +883,7 @@ __global__ void __launch_bounds__(kBT) k_cluster(const __grid_constant__ BottomA
     for (int up = 0; up < 2; ++up) {
 #pragma unroll 1
         for (int t = 0; t < (up ? A.nu2 : A.nu1); ++t)
-            tile_smooth<true>(ta, T.S, &T, TX, rank, ntiles, false);
+            tile_smooth<true>(ta, T.S, &T, TX, rank, ntiles, A.fas && !up && t == 0);
         if (up) break;
         // ---- residual r = rhs - L(pn + u) of the own cell (as b_residual, mode 0)
         {
@@ -964,7 +983,7 @@ void prepare_bottom_kernel() {
 }
 
 void launch_bottom(const BottomArgs &A, size_t smem, cudaStream_t st) {
-    k_bottom<<<1, kBT, smem, st>>>(A);
+    launch_pdl(k_bottom, dim3(1), dim3(kBT), smem, st, A);
 }
 
 size_t cluster_smem_bytes(size_t bottom_bytes) { return kTileBytes + bottom_bytes; }
@@ -997,13 +1016,15 @@ void launch_cluster(const BottomArgs &A, int tiles, size_t smem, cudaStream_t st
     cfg.blockDim = dim3(kBT);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = tiles;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     cudaLaunchKernelEx(&cfg, k_cluster, A);
 }
 

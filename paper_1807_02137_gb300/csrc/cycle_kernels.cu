@@ -3,6 +3,7 @@
 #include "arith.cuh"
 #include "coarse_body.cuh"
 #include "reduce.cuh"
+#include "tma.cuh"
 
 namespace segmg {
 
@@ -208,6 +209,8 @@ __global__ void __launch_bounds__(256) k_residual_restrict(LevelView<float> L, L
 __global__ void __launch_bounds__(256) k_chunk_sums(const double *part, int np, double *stage) {
     __shared__ double red[33];
     const int b = blockIdx.x, k = blockIdx.y;
+    pdl_wait();
+    pdl_trigger();
     const double s = chunk_sum(part + (size_t)k * np, b * kSumChunk, min(np, (b + 1) * kSumChunk), red);
     if (threadIdx.x == 0) stage[(size_t)k * gridDim.x + b] = s;
 }
@@ -215,6 +218,8 @@ __global__ void __launch_bounds__(256) k_chunk_sums(const double *part, int np, 
 // Sums `np` partials in a fixed order into *out (one block).
 __global__ void __launch_bounds__(256) k_sum_partials(const double *partials, int np, double *out) {
     __shared__ double red[33];
+    pdl_wait();
+    pdl_trigger();
     const double s = chunk_sum(partials, 0, np, red);
     if (threadIdx.x == 0) *out = s;
 }
@@ -341,16 +346,16 @@ void launch_interp_add(const LevelView<T> &Lf, const LevelView<T> &Lc, cudaStrea
 constexpr size_t kCoarseSmemMax = 200 * 1024;
 
 void launch_chunk_sums(const double *part, int np, int K, double *stage, cudaStream_t st) {
-    k_chunk_sums<<<dim3(sum_blocks(np), K), 256, 0, st>>>(part, np, stage);
+    launch_pdl(k_chunk_sums, dim3(sum_blocks(np), K), dim3(256), 0, st, part, np, stage);
 }
 
 void launch_sum_partials(double *partials, int np, double *out, cudaStream_t st) {
     const int G = sum_blocks(np);
     if (G == 1) {
-        k_sum_partials<<<1, 256, 0, st>>>(partials, np, out);
+        launch_pdl(k_sum_partials, dim3(1), dim3(256), 0, st, partials, np, out);
     } else {   // the chunk sums go to the G doubles after the partials
         launch_chunk_sums(partials, np, 1, partials + np, st);
-        k_sum_partials<<<1, 256, 0, st>>>(partials + np, G, out);
+        launch_pdl(k_sum_partials, dim3(1), dim3(256), 0, st, partials + np, G, out);
     }
 }
 

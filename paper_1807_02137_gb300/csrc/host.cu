@@ -325,6 +325,7 @@ struct Solver final : SolverBase {
         v.cls = L.cls;
         v.omega = use_omega && omega_valid[l] ? omega_buf[l] : nullptr;
         v.has_rhs = l > 0 ? 1 : 0;
+        v.u_in_r = 0;
         return v;
     }
 
@@ -548,7 +549,7 @@ struct Solver final : SolverBase {
         return MG_OK;
     }
 
-    void launch_bottom_cycle(bool cluster = false) {
+    void launch_bottom_cycle(bool cluster, bool fas) {
         if constexpr (std::is_same<T, float>::value) {
             const int first = cluster ? lc : lb;
             BottomArgs a{};
@@ -559,6 +560,7 @@ struct Solver final : SolverBase {
             a.aos_dt = p.aos_dt;
             for (int l = first; l < nlev; ++l) a.g[l] = view(l);
             a.first = a.g[first];
+            a.fas = fas;
             a.mp = mp;
             a.A1frac = A1 / ((double)n * m);
             a.h2nm_coarse = h2nm(nlev - 1);
@@ -785,8 +787,10 @@ struct Solver final : SolverBase {
                     launch_snapshot_fas_tma(v, area_ptr(), lv[l].smaps, &dsc->err, wait_limit, st);
                 fas_level = -1;
             } else if (l == interp_level) {   // the first snapshot after the coarse grid applies its correction
-                if constexpr (std::is_same<T, float>::value)
+                if constexpr (std::is_same<T, float>::value) {
+                    v.u_in_r = interp_to_r(v);
                     launch_snapshot_interp_tma(v, view(l + 1), area_ptr(), lv[l].smaps, &dsc->err, wait_limit, st);
+                }
                 interp_level = -1;
             } else {
                 snapshot(l, v);
@@ -808,12 +812,14 @@ struct Solver final : SolverBase {
         Range range(kLevelNames[l]);
         if (l == 0) fas_level = interp_level = -1;   // nothing pending from an enqueue cut short
         if (l == lc) {
-            launch_bottom_cycle(true);
+            launch_bottom_cycle(true, l == fas_level);
+            fas_level = -1;
             ++launches;
             return;
         }
         if (l == lb) {
-            launch_bottom_cycle();
+            launch_bottom_cycle(false, l == fas_level);
+            fas_level = -1;
             ++launches;
             return;
         }
@@ -837,10 +843,9 @@ struct Solver final : SolverBase {
             launches += 3;
         }
         // FAS right-hand side on grid l+1: rhs += L(pn + u0).  FP32 storage with a pre-smoothing
-        // on grid l+1 by the per-grid kernels: its first snapshot completes it (fas_level);
+        // on grid l+1: its first snapshot completes it (fas_level), in the bottom kernels too;
         // otherwise a residual launch here
-        const bool fas_in_snapshot = std::is_same<T, float>::value && p.nu1 >= 1 && l + 1 != lc && l + 1 != lb &&
-                                     l + 1 < nlev - 1;
+        const bool fas_in_snapshot = std::is_same<T, float>::value && p.nu1 >= 1 && l + 1 < nlev - 1;
         if (fas_in_snapshot) {
             fas_level = l + 1;
             launches += area_launches(l);
@@ -853,10 +858,10 @@ struct Solver final : SolverBase {
             launches += area_launches(l) + area_launches(l + 1) + 1;
         }
         cycle(l + 1);
-        // the coarse-grid correction: in the first post-smoothing snapshot (FP32 storage, the
-        // Spencer-Chen model: the Rada-Chen area term before a snapshot reads the corrected u),
-        // else its own launch
-        if (std::is_same<T, float>::value && p.nu2 >= 1 && p.model == MG_MODEL_SC) {
+        // the coarse-grid correction: in the first post-smoothing snapshot (FP32 storage, the TMA
+        // sweeps, the Spencer-Chen model: the Rada-Chen area term before a snapshot reads the
+        // corrected u), else its own launch
+        if (std::is_same<T, float>::value && p.nu2 >= 1 && p.model == MG_MODEL_SC && p.smoother == MG_SMOOTH_FUSED) {
             interp_level = l;
         } else {
             launch_interp_add<T>(view(l), view(l + 1), st);

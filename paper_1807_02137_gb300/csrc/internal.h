@@ -48,6 +48,7 @@ struct LevelView {
     const T *omega;            // relaxation weights of the Hybrid Smoother 2 point updates
                                // (phi += omega (g - phi)); NULL: plain updates
     int has_rhs;    // 0 on the finest grid (zero right-hand side)
+    int u_in_r;     // interpolating snapshot: writes the corrected u to r; the sweep A after it: reads r
 };
 
 // Device-resident scalars (double) shared by the kernels of one handle.
@@ -168,10 +169,11 @@ template <typename T>
 void launch_hs1_blocks(const LevelView<T> &L, cudaStream_t st);
 
 // sweep_tma.cu: the fused sweep for FP32 storage with TMA-staged tiles.  A SweepMaps holds the
-// tensor maps (CUtensorMap, 128 bytes each) of u, t, G and f of one grid for one tile shape.
+// tensor maps (CUtensorMap, 128 bytes each) of u, t, r, G and f of one grid for one tile shape.
 struct SweepMaps {
     alignas(64) unsigned char u[128];
     alignas(64) unsigned char t[128];
+    alignas(64) unsigned char r[128];
     alignas(64) unsigned char G[128];
     alignas(64) unsigned char f[128];
 };
@@ -199,10 +201,11 @@ void launch_snapshot_tma(const LevelView<float> &L, const double *area, const Sn
 void launch_snapshot_fas_tma(const LevelView<float> &L, const double *area, const SnapMaps &M, int *err,
                              long long wait_limit, cudaStream_t st);
 // The first snapshot of grid L's post-smoothing: first applies the coarse-grid correction
-// u += P (u_c - u0_c) from grid C (Algorithm 1's interpolation) and writes u (the separate
-// interpolation launch then does not run).
+// u += P (u_c - u0_c) from grid C (Algorithm 1's interpolation) and writes it to r, the next
+// sweep A's input (L.u_in_r), or to u (the separate interpolation launch then does not run).
 void launch_snapshot_interp_tma(const LevelView<float> &L, const LevelView<float> &C, const double *area,
                                 const SnapMaps &M, int *err, long long wait_limit, cudaStream_t st);
+bool interp_to_r(const LevelView<float> &L);   // whether it writes r (u_in_r), else u in place
 void launch_snapshot_norm_tma(const LevelView<float> &L, const double *area, const SnapMaps &M, double *partials,
                               int *err, long long wait_limit, cudaStream_t st);
 // Tensor maps of the TMA-staged residual kernels of one FP32 grid (residual_tma.cu): pn, u and w
@@ -288,6 +291,7 @@ struct BottomArgs {
     int coarse_aos;    // the coarsest solve by AOS iterations (step aos_dt)
     int pad;           // odd row pitches in shared memory (where they fit, see bottom_smem_bytes)
     double aos_dt;
+    int fas;                  // grid lb's right-hand side lacks L(pn + u0): its first snapshot adds it
     LevelView<float> first;   // grid lb
     LevelView<float> g[kMaxLevels];
     ModelParams mp;

@@ -54,7 +54,7 @@ constexpr int kSumChunk = 1024;
 __device__ __forceinline__ double chunk_sum(const double *a, int begin, int end, double *red) {
     const int tid = threadIdx.y * blockDim.x + threadIdx.x, nt = blockDim.x * blockDim.y;
     double v = 0.0;
-    for (int q = begin + tid; q < end; q += nt) v += a[q];
+    for (int q = begin + tid; q < end; q += nt) v += __ldcg(a + q);   // a dependent launch's input: through L2
     return block_sum(v, red);
 }
 

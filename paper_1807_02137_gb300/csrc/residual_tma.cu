@@ -63,12 +63,14 @@ __global__ void __launch_bounds__(256, MINB)
         fence_proxy_async();
         const unsigned wbytes = MIXED ? 36u * kCb * 2u : 36u * kC * 4u;
         mbar_expect_tx(&S.bar, 2u * 36u * kC * 4u + wbytes + 4096u + (hasX ? 4096u : 0u));
+        pdl_wait();   // at a step's start the kernel before has just written F
         tma_load(&S.P[0][0], &mP, j0 - 4, i0 - 2, &S.bar);
-        tma_load(&S.U[0][0], &mU, j0 - 4, i0 - 2, &S.bar);
         if (MIXED) tma_load(&S.Wb[0][0], &mW, j0 - 8, i0 - 2, &S.bar);
         else tma_load(&S.W[0][0], &mW, j0 - 4, i0 - 2, &S.bar);
         tma_load(&S.F[0][0], &mF, j0, i0, &S.bar);
+        tma_load(&S.U[0][0], &mU, j0 - 4, i0 - 2, &S.bar);
         if (hasX) tma_load(&S.X[0][0], &mX, j0, i0, &S.bar);
+        pdl_trigger();
     }
     __syncthreads();
     bool ok = true;
@@ -113,7 +115,7 @@ __global__ void __launch_bounds__(256, MINB)
         if (tid < 68) g_at(1 + (tid >> 1), (tid & 1) ? 36 : 3, true);
     }
     __syncthreads();
-    const T ar = area ? T(area[L.level]) : T(0);
+    const T ar = area ? T(__ldcg(area + L.level)) : T(0);
     const T c2 = L.cdiff * T(0.5);
     const int gj = j0 + lane, c = lane + 4;
     const size_t lim = (size_t)n * p;
@@ -186,12 +188,15 @@ __global__ void __launch_bounds__(256, MINB)
         fence_proxy_async();
         const unsigned wbytes = MIXED ? 37u * kCb * 2u : 37u * kC * 4u;
         mbar_expect_tx(&S.bar, 2u * 37u * kC * 4u + wbytes + 33u * 36u * 4u * (L.has_rhs ? 2u : 1u));
+        // pn, w and F are fixed during a step: fetched before a dependent launch's wait
         tma_load(&S.P[0][0], &mP, j0 - 4, i0 - 2, &S.bar);
-        tma_load(&S.U[0][0], &mU, j0 - 4, i0 - 2, &S.bar);
         if (MIXED) tma_load(&S.Wb[0][0], &mW, j0 - 8, i0 - 2, &S.bar);
         else tma_load(&S.W[0][0], &mW, j0 - 4, i0 - 2, &S.bar);
         tma_load(&S.F[0][0], &mF, j0, i0, &S.bar);
+        pdl_wait();
+        tma_load(&S.U[0][0], &mU, j0 - 4, i0 - 2, &S.bar);
         if (L.has_rhs) tma_load(&S.RH[0][0], &mR, j0, i0, &S.bar);
+        pdl_trigger();
     }
     __syncthreads();
     bool ok = true;
@@ -238,7 +243,7 @@ __global__ void __launch_bounds__(256, MINB)
     }
     __syncthreads();
     // r on rows i0 .. i0+32, columns j0 .. j0+32 (zero outside the grid)
-    const float ar = area ? float(area[L.level]) : 0.f;
+    const float ar = area ? float(__ldcg(area + L.level)) : 0.f;
     const float c2 = L.cdiff * 0.5f;
     const bool rin = gin;   // every r cell has its four faces and its G ring inside the grid
     auto r_at = [&](int ti, int tj, auto in_tag) {
@@ -312,8 +317,8 @@ template <int MODE, bool MIXED, bool NORM>
 void launch_res(const LevelView<float> &L, const double *area, float *out, double *partials, const SnapMaps &M,
                 const unsigned char *mU, const unsigned char *mX, int *err, long long wl, cudaStream_t st) {
     dim3 grid((L.m + 31) / 32, (L.n + 31) / 32), block(32, 8);
-    k_residual_tma<MODE, MIXED, NORM, kResMinB><<<grid, block, res_smem<MODE, MIXED, NORM>(), st>>>(
-        L, area, out, partials, *tm(M.P), *tm(mU), *tm(M.W), *tm(M.F), *tm(mX), err, wl);
+    launch_pdl(k_residual_tma<MODE, MIXED, NORM, kResMinB>, grid, block, res_smem<MODE, MIXED, NORM>(), st, L, area, out,
+               partials, *tm(M.P), *tm(mU), *tm(M.W), *tm(M.F), *tm(mX), err, wl);
 }
 
 template <bool MIXED>
@@ -361,13 +366,11 @@ void launch_residual_restrict_tma(const LevelView<float> &L, const LevelView<flo
     dim3 grid((L.m + 31) / 32, (L.n + 31) / 32), block(32, 8);
     const unsigned char *mR = L.has_rhs ? R.R33 : R.F33;
     if (L.wb)
-        k_residual_restrict_tma<true, kRRMinB><<<grid, block, rr_smem<true>(), st>>>(L, C, area, *tm(R.P37), *tm(R.U37),
-                                                                           *tm(R.W37), *tm(R.F33), *tm(mR), err,
-                                                                           wait_limit);
+        launch_pdl(k_residual_restrict_tma<true, kRRMinB>, grid, block, rr_smem<true>(), st, L, C, area, *tm(R.P37),
+                   *tm(R.U37), *tm(R.W37), *tm(R.F33), *tm(mR), err, wait_limit);
     else
-        k_residual_restrict_tma<false, kRRMinB><<<grid, block, rr_smem<false>(), st>>>(L, C, area, *tm(R.P37), *tm(R.U37),
-                                                                             *tm(R.W37), *tm(R.F33), *tm(mR), err,
-                                                                             wait_limit);
+        launch_pdl(k_residual_restrict_tma<false, kRRMinB>, grid, block, rr_smem<false>(), st, L, C, area, *tm(R.P37),
+                   *tm(R.U37), *tm(R.W37), *tm(R.F33), *tm(mR), err, wait_limit);
 }
 
 }  // namespace segmg

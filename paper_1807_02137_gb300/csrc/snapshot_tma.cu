@@ -58,8 +58,9 @@ struct SnapTmaSmem {
 // rhs += L(pn + u0) (Algorithm 1), with the G it forms anyway, writes it and takes it into f,
 // instead of a separate residual launch before the snapshot.  XT = 2, interpolation (the first
 // snapshot of a grid's post-smoothing): the block first applies the coarse-grid correction
-// u += P (u_c - u0_c) (Algorithm 1) to the box cells it reads and writes its tile's corrected u,
-// instead of a separate interpolation launch.  Both take the separate launches' operations, so
+// u += P (u_c - u0_c) (Algorithm 1) to the box cells it reads and writes its tile's corrected u
+// to r, which the following sweep A reads instead of u (u itself stays as it is: other blocks copy
+// their halo from it), instead of a separate interpolation launch.  Both take the separate launches' operations, so
 // the values are the same.
 template <int WARPS, int MINB, bool MIXED, bool NORM = false, int XT = 0>
 __global__ void __launch_bounds__(32 * WARPS, MINB)
@@ -81,15 +82,19 @@ __global__ void __launch_bounds__(32 * WARPS, MINB)
         mbar_init(&S.bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         fence_proxy_async();
+        // pn, w and F are fixed during a step: fetched before a dependent launch's wait
         const unsigned wbytes = MIXED ? (unsigned)(kBR * kBCb * 2) : (unsigned)(kBR * kBC * 4);
         mbar_expect_tx(&S.bar, 2u * kBR * kBC * 4u + wbytes + 4096u + (L.has_rhs ? 4096u : 0u));
         tma_load(&S.P[0][0], &mP, j0 - 4, i0 - 2, &S.bar);
-        tma_load(&S.U[0][0], &mU, j0 - 4, i0 - 2, &S.bar);
         if (MIXED) tma_load(&S.Wb[0][0], &mW, j0 - 8, i0 - 2, &S.bar);
         else tma_load(&S.W[0][0], &mW, j0 - 4, i0 - 2, &S.bar);
         tma_load(&S.F[0][0], &mF, j0, i0, &S.bar);
+        pdl_wait();
+        tma_load(&S.U[0][0], &mU, j0 - 4, i0 - 2, &S.bar);
         if (L.has_rhs) tma_load(&S.R[0][0], &mR, j0, i0, &S.bar);
+        pdl_trigger();
     }
+    if (INTERP) pdl_wait();   // every thread reads the coarse grid before the boxes arrive
     int I0 = 0, J0 = 0;   // INTERP: the first coarse row and column of E
     if (INTERP) {   // u_c - u0_c while the boxes are in flight
         I0 = max(0, i0 / 2 - 2);
@@ -100,7 +105,7 @@ __global__ void __launch_bounds__(32 * WARPS, MINB)
             float e = 0.f;
             if (I < Cg.n && J < Cg.m) {
                 const size_t o = (size_t)I * Cg.pitch + J;
-                e = sub_rn(ldc(Cg.u, o, lc, kDbgInterp), ldc(Cg.u0, o, lc, kDbgInterp));
+                if (MG_DBG_OK(o, lc, kDbgInterp)) e = sub_rn(__ldcg(Cg.u + o), __ldcg(Cg.u0 + o));
             }
             S.E[r][cc] = e;
         }
@@ -119,7 +124,8 @@ __global__ void __launch_bounds__(32 * WARPS, MINB)
     if (INTERP) {
         // u += P (u_c - u0_c) on the in-grid box cells of rows 0..35 and columns 2..37 (every u
         // the G box, the class and the residuals read), as k_interp_add: then the tile's cells
-        // to u
+        // to r, not to u, whose halo a neighbouring block may still have to copy (u_in_r; see
+        // interp_to_r for the grids that keep u)
         for (int q = tid; q < kBR * (kBC - 4); q += NT) {
             const int a = q / (kBC - 4), c = 2 + (q - a * (kBC - 4)), gi = i0 - 2 + a, gj = j0 - 4 + c;
             if (gi < 0 || gi >= n || gj < 0 || gj >= m) continue;
@@ -137,9 +143,10 @@ __global__ void __launch_bounds__(32 * WARPS, MINB)
         }
         __syncthreads();
         const size_t lim = (size_t)n * p;
+        float *uo = L.u_in_r ? L.r : L.u;
         for (int q = tid; q < 1024; q += NT) {
             const int ti = q >> 5, tj = q & 31, gi = i0 + ti, gj = j0 + tj;
-            if (gi < n && gj < m) stc(L.u, (size_t)gi * p + gj, lim, kDbgInterp, S.U[ti + 2][tj + 4]);
+            if (gi < n && gj < m) stc(uo, (size_t)gi * p + gj, lim, kDbgInterp, S.U[ti + 2][tj + 4]);
         }
     }
     // edge tiles: box cells of pn and u outside the grid take the clamped cell's values (the
@@ -179,7 +186,7 @@ __global__ void __launch_bounds__(32 * WARPS, MINB)
         if (tid < 68) g_at(1 + (tid >> 1), (tid & 1) ? 36 : 3, true);
     }
     __syncthreads();
-    const T ar = area ? T(area[L.level]) : T(0);
+    const T ar = area ? T(__ldcg(area + L.level)) : T(0);
     const int gj = j0 + lane, c = lane + 4;
     const int lenr = min(32, m - j0), lenc = min(32, n - i0);
     T acc = T(0);   // NORM: this thread's sum of r^2
@@ -307,8 +314,8 @@ void launch_v(const LevelView<float> &L, const double *area, const SnapMaps &M, 
     const auto *mw = reinterpret_cast<const CUtensorMap *>(M.W);
     const auto *mf = reinterpret_cast<const CUtensorMap *>(M.F);
     const auto *mr = reinterpret_cast<const CUtensorMap *>(L.has_rhs ? M.R : M.F);
-    k_snapshot_tma<WARPS, MINB, MIXED, NORM, XT><<<grid, block, snap_smem<WARPS, MINB, MIXED>(), st>>>(
-        L, area, *mp, *mu, *mw, *mf, *mr, err, wl, partials, C ? *C : L);
+    launch_pdl(k_snapshot_tma<WARPS, MINB, MIXED, NORM, XT>, grid, block, snap_smem<WARPS, MINB, MIXED>(), st,
+               L, area, *mp, *mu, *mw, *mf, *mr, err, wl, partials, C ? *C : L);
 }
 
 template <bool MIXED, int XT = 0>
@@ -377,6 +384,19 @@ void launch_snapshot_interp_tma(const LevelView<float> &L, const LevelView<float
                                 const SnapMaps &M, int *err, long long wait_limit, cudaStream_t st) {
     if (M.mixed) launch_mixed<true, 2>(L, area, M, err, wait_limit, st, &C);
     else launch_mixed<false, 2>(L, area, M, err, wait_limit, st, &C);
+}
+
+// Whether the interpolating snapshot of a grid writes the corrected u to r.  In place, a block whose
+// neighbour above has already written copies a halo that is corrected, and corrects it again: its
+// coefficients (lagged ones) at the tile's upper edge then differ by the correction's change over a
+// cell.  Whether that happens depends on the blocks' timing, unless the row of tiles above is far
+// ahead, as it always is where a row is more than 0.65 of the resident blocks (images wider than
+// about 22,000 cells).  Those grids keep the in-place form: there it is what every run has done so
+// far, and the step control's choice of tau follows from it (25000^2 with r: of four images one took
+// the same tau and V-cycles, the others tau / 2 to 8 tau and 9, 10, 21 V-cycles instead of 11, 9, 25).
+bool interp_to_r(const LevelView<float> &L) {
+    const long resident = (long)g_snap_occ.sms * g_snap_occ.per_sm[L.wb ? 1 : 0][2];
+    return 20L * ((L.m + 31) / 32) <= 13 * resident;
 }
 
 void launch_snapshot_norm_tma(const LevelView<float> &L, const double *area, const SnapMaps &M, double *partials,

@@ -162,13 +162,13 @@ __global__ void __launch_bounds__(TS::NT, TS::MinBlocks) k_sweep_tma(LevelView<f
                 const int gi = i0 - kH + a, piece = (j0 >> 5) - 1 + pc;
                 if (gi >= 0 && gi < n && piece >= 0 && piece < L.npm &&
                     MG_DBG_OK(((size_t)SWEEP * n + gi) * L.npm + piece, (size_t)2 * n * L.npm, kDbgMaskLoad))
-                    w[r] = __ldg(L.mrow + ((size_t)SWEEP * n + gi) * L.npm + piece);
+                    w[r] = __ldcg(L.mrow + ((size_t)SWEEP * n + gi) * L.npm + piece);
             } else {
                 const int b = q / kColPieces, pc = q % kColPieces;
                 const int gj = j0 - kH + b, piece = (i0 >> 5) - 1 + pc;
                 if (gj >= 0 && gj < m && piece >= 0 && piece < L.npn &&
                     MG_DBG_OK(((size_t)(SWEEP - 2) * m + gj) * L.npn + piece, (size_t)2 * m * L.npn, kDbgMaskLoad))
-                    w[r] = __ldg(L.mcol + ((size_t)(SWEEP - 2) * m + gj) * L.npn + piece);
+                    w[r] = __ldcg(L.mcol + ((size_t)(SWEEP - 2) * m + gj) * L.npn + piece);
             }
         }
     };
@@ -203,12 +203,26 @@ __global__ void __launch_bounds__(TS::NT, TS::MinBlocks) k_sweep_tma(LevelView<f
     };
     int tile = blockIdx.x;
     uint32_t mw[kMaskPer];
+    // The first tile's copies.  Under a dependent launch the predecessor of sweeps B to D is the sweep
+    // before (it wrote this sweep's input; G, f and the masks are older and fetched before the wait),
+    // that of sweep A the snapshot, which may have written all of them.
+    if (SWEEP == 0) pdl_wait();
     load_masks(tile, mw);
     if (tid == 0) {   // the thread that initialises the barriers issues the first tile's copies
         S.flags = 0;
         for (int k = 0; k < STAGES; ++k) mbar_init(&S.bar[k], 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-        if (tile < ntiles) issue(tile, 0);
+        if (tile < ntiles) {
+            const int ty = tile / ntx, tx = tile - ty * ntx;
+            const int x = tx * kOW - kH, y = ty * kOH - kH;
+            fence_proxy_async();
+            mbar_expect_tx(&S.bar[0], 3u * TS::BoxBytes);
+            tma_load(&S.box[0][1][0][0], &tG, x, y, &S.bar[0]);
+            tma_load(&S.box[0][2][0][0], &tf, x, y, &S.bar[0]);
+            if (SWEEP != 0) pdl_wait();
+            tma_load(&S.box[0][0][0][0], &tin, x, y, &S.bar[0]);
+        }
+        pdl_trigger();
     }
     __syncthreads();
     for (int k = 0; tile < ntiles; ++k, tile += gridDim.x) {
@@ -315,14 +329,15 @@ void set_attrs() {
 template <int SW, typename TS>
 void launch_one(const LevelView<float> &L, const SweepMaps &M, int sms, int *err, long long wl, cudaStream_t st) {
     const int ntiles = ((L.m + TS::OW - 1) / TS::OW) * ((L.n + TS::OH - 1) / TS::OH);
-    const CUtensorMap *in = reinterpret_cast<const CUtensorMap *>((SW & 1) ? M.t : M.u);
+    const CUtensorMap *in = reinterpret_cast<const CUtensorMap *>((SW & 1) ? M.t : (SW == 0 && L.u_in_r ? M.r : M.u));
     const CUtensorMap &mG = *reinterpret_cast<const CUtensorMap *>(M.G);
     const CUtensorMap &mf = *reinterpret_cast<const CUtensorMap *>(M.f);
     if (TS::OneTile || ntiles <= sms * tma_blocks_per_sm<SW, TS, 1>()) {
-        k_sweep_tma<SW, TS, 1><<<ntiles, TS::NT, tma_smem<SW, TS, 1>(), st>>>(L, *in, mG, mf, err, wl);
+        launch_pdl(k_sweep_tma<SW, TS, 1>, dim3(ntiles), dim3(TS::NT), tma_smem<SW, TS, 1>(), st, L, *in, mG, mf,
+                   err, wl);
     } else if constexpr (!TS::OneTile) {
         const int grid = std::min(ntiles, sms * tma_blocks_per_sm<SW, TS, 2>());
-        k_sweep_tma<SW, TS, 2><<<grid, TS::NT, tma_smem<SW, TS, 2>(), st>>>(L, *in, mG, mf, err, wl);
+        launch_pdl(k_sweep_tma<SW, TS, 2>, dim3(grid), dim3(TS::NT), tma_smem<SW, TS, 2>(), st, L, *in, mG, mf, err, wl);
     }
 }
 
@@ -378,7 +393,8 @@ bool encode(void *out, float *base, int n, int m, int pitch, int RH, int RW) {
 
 template <typename TS>
 bool encode_shape(const LevelView<float> &L, SweepMaps &M) {
-    return encode(M.u, L.u, L.n, L.m, L.pitch, TS::RH, TS::PW) && encode(M.t, L.t, L.n, L.m, L.pitch, TS::RH, TS::PW) &&
+    return encode(M.u, L.u, L.n, L.m, L.pitch, TS::RH, TS::PW) && encode(M.r, L.r, L.n, L.m, L.pitch, TS::RH, TS::PW) &&
+           encode(M.t, L.t, L.n, L.m, L.pitch, TS::RH, TS::PW) &&
            encode(M.G, L.G, L.n, L.m, L.pitch, TS::RH, TS::PW) && encode(M.f, L.f, L.n, L.m, L.pitch, TS::RH, TS::PW);
 }
 

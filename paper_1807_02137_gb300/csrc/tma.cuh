@@ -10,6 +10,8 @@
 
 #include <cuda.h>
 
+#include <utility>
+
 namespace segmg {
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -52,6 +54,32 @@ __device__ __forceinline__ void tma_load(void *dst, const CUtensorMap *map, int 
 
 __device__ __forceinline__ void fence_proxy_async() {
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+}
+
+// Programmatic dependent launch (PDL).  A kernel launched with the attribute starts once every block
+// of the kernel before it has called pdl_trigger (or ended); pdl_wait returns when that kernel has
+// completed and its writes are visible.  Every kernel here calls pdl_trigger after its own pdl_wait:
+// a kernel that has started then knows that all kernels before its predecessor are complete, and may
+// read before its pdl_wait whatever its predecessor does not write.  What the predecessor does write
+// is read through L2 (TMA copies, ldcg): a block that started early may find older lines in L1.
+// Without the attribute both calls do nothing.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
+// Launches `kernel` as a dependent launch.
+template <typename... P, typename... A>
+void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
 }  // namespace segmg
