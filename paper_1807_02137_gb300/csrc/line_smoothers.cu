@@ -3,9 +3,9 @@
 //
 // GSLINE-I: every column is one tridiagonal system (eq. system) coupling the column's cells
 // through A and B, with C and D terms from the current values.  The columns of one parity are
-// not neighbours, so all even columns are solved at once, then all odd ones (zebra); one thread
-// solves one whole column by the Thomas algorithm, streaming down the rows, with the eliminated
-// diagonal and right-hand side kept in two scratch grids.
+// not neighbours, so all even columns are solved at once, then all odd ones (zebra), each by the
+// Thomas algorithm down and up its rows, with the eliminated diagonal (its reciprocal in FP32) and
+// right-hand side kept in two scratch grids.
 //
 // Hybrid Smoother 1: after GSLINE-I, every cell P of the set D (from the coefficient snapshot:
 // class byte = 1 << index of the smallest coefficient) and its neighbours other than the lagged
@@ -23,90 +23,126 @@ namespace segmg {
 namespace {
 
 // ---------------------------------------------------------------------------------------
-// GSLINE-I, one parity of columns.  dg / rg: scratch for the eliminated diagonal and
-// right-hand side of every cell of the column (pitched like the grid).
+// GSLINE-I, one parity of columns: a block solves 32 of them.
+//
+// A column's elimination and substitution are serial recurrences, and a grid has few columns (512
+// of a parity at 1024^2): the recurrence's chain sets the time, about 45 cycles a row down (a
+// reciprocal, a product, a multiply-add) and 12 up, if nothing else stands in it.  So one warp
+// runs the 32 recurrences from values in shared memory, and the block's other warps form those
+// values (faces, products, right-hand sides) and store the results, a chunk of kGR rows ahead and
+// behind.  (One thread a column that also loaded and formed its values took about 250 cycles a row
+// each way: 4.2 ms a V-cycle at 1024^2.)
+// dg / rg: scratch for what the eliminated rows leave (the reciprocal of the diagonal, or in FP64 the
+// diagonal, and the right-hand side), row by row at the columns' own order (pitched like the grid).
 // ---------------------------------------------------------------------------------------
+constexpr int kGW = 8;     // warps: the solving one and seven that form values
+
 template <typename T>
-__global__ void __launch_bounds__(128) k_gsline(LevelView<T> L, int parity, T *__restrict__ dg, T *__restrict__ rg) {
-    constexpr int R = 8;   // rows whose inputs are loaded together before their recurrence steps
-    const int j = parity + 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+__global__ void __launch_bounds__(32 * kGW) k_gsline(LevelView<T> L, int parity, T *__restrict__ dg, T *__restrict__ rg) {
+    constexpr int kGR = 128 / sizeof(T);   // rows of a chunk (32 KB of values in two chunks)
+    // down: lo, up, diagonal, right-hand side; up: up, reciprocal, right-hand side
+    __shared__ T val[2][4][kGR][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n = L.n, m = L.m, p = L.pitch;
-    if (j >= m) return;
-    const bool hE = j + 1 < m, hW = j > 0;
-    const T *__restrict__ G = L.G;
-    const T *__restrict__ U = L.u;   // the neighbouring columns (the other parity) are only read
-    const T *__restrict__ F = L.f;
-    T cup_prev = T(0), cdi_prev = T(1), crh_prev = T(0);
-    T g_next = __ldg(G + j);           // G of the row after the previous chunk's last row
-    for (int i0 = 0; i0 < n; i0 += R) {
-        T g[R + 1], gE[R], gW[R], uE[R], uW[R], f[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int i = i0 + r;
-            if (i < n) {
-                const size_t o = (size_t)i * p + j;
-                gE[r] = __ldg(G + (hE ? o + 1 : o));
-                gW[r] = __ldg(G + (hW ? o - 1 : o));
-                uE[r] = __ldg(U + (hE ? o + 1 : o));
-                uW[r] = __ldg(U + (hW ? o - 1 : o));
-                f[r] = __ldg(F + o);
-                g[r + 1] = i + 1 < n ? __ldg(G + o + p) : T(0);
-            }
-        }
-        g[0] = g_next;
-        T g_up = i0 > 0 ? __ldg(G + (size_t)(i0 - 1) * p + j) : T(0);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int i = i0 + r;
+    const int c = blockIdx.x * 32 + lane, j = parity + 2 * c;   // this lane's column
+    const bool on = j < m;
+    const int jc = on ? j : parity;                             // a lane past the last column reads the first
+    const bool hE = jc + 1 < m, hW = jc > 0;
+    const int chunks = (n + kGR - 1) / kGR;
+    const size_t lim = (size_t)n * p;
+    // the coefficients and the right-hand side of rows i0 .. i0 + kGR - 1 into val[b]
+    auto form = [&](int k, int b) {
+        for (int r = warp - 1; r < kGR; r += kGW - 1) {
+            const int i = k * kGR + r;
             if (i >= n) break;
-            const size_t o = (size_t)i * p + j;
-            const T gc = g[r];
-            const T aS = face(gc, g[r + 1], i + 1 < n), aN = face(gc, g_up, i > 0);
-            const T aE = face(gc, gE[r], hE), aW = face(gc, gW[r], hW);
-            const T lo = mul_rn(L.cdiff, aN), up = mul_rn(L.cdiff, aS);
+            const size_t o = (size_t)i * p + jc;
+            const bool hS = i + 1 < n, hN = i > 0;
+            const T gc = __ldg(L.G + o);
+            const T aS = face(gc, hS ? __ldg(L.G + o + p) : T(0), hS), aN = face(gc, hN ? __ldg(L.G + o - p) : T(0), hN);
+            const T aE = face(gc, hE ? __ldg(L.G + o + 1) : T(0), hE), aW = face(gc, hW ? __ldg(L.G + o - 1) : T(0), hW);
+            const T uE = hE ? __ldg(L.u + o + 1) : __ldg(L.u + o), uW = hW ? __ldg(L.u + o - 1) : __ldg(L.u + o);
             const T sum = add_rn(add_rn(aN, aS), add_rn(aE, aW));
-            T di = -fma_rn(L.cdiff, sum, L.inv_tau);
-            const T across = fma_rn(aW, uW[r], mul_rn(aE, uE[r]));
-            T rhs = fma_rn(-L.cdiff, across, f[r]);
-            if (i > 0) {
-                const T wgt = div_relax(lo, cdi_prev);
-                di = fma_rn(-wgt, cup_prev, di);
-                rhs = fma_rn(-wgt, crh_prev, rhs);
-            }
-            stc(dg, o, (size_t)n * p, kDbgOther, di);
-            stc(rg, o, (size_t)n * p, kDbgOther, rhs);
-            cup_prev = up;
-            cdi_prev = di;
-            crh_prev = rhs;
-            g_up = gc;
+            const T across = fma_rn(aW, uW, mul_rn(aE, uE));
+            val[b][0][r][lane] = mul_rn(L.cdiff, aN);
+            val[b][1][r][lane] = mul_rn(L.cdiff, aS);
+            val[b][2][r][lane] = -fma_rn(L.cdiff, sum, L.inv_tau);
+            val[b][3][r][lane] = fma_rn(-L.cdiff, across, __ldg(L.f + o));
         }
-        g_next = g[R < n - i0 ? R : n - i0];
+    };
+    // ---- elimination, downwards
+    if (warp > 0) form(0, 0);
+    __syncthreads();
+    T up_prev = T(0), rec_prev = T(0), rhs_prev = T(0);
+    for (int k = 0; k < chunks; ++k) {
+        const int b = k & 1, rows = min(kGR, n - k * kGR);
+        if (warp > 0) {
+            if (k + 1 < chunks) form(k + 1, b ^ 1);
+        } else {
+            for (int r0 = 0; r0 < rows; r0 += 8) {
+                T lo[8], up[8], di[8], rh[8];
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {   // (rows past the grid's last are read and not used)
+                    lo[r] = val[b][0][r0 + r][lane]; up[r] = val[b][1][r0 + r][lane];
+                    di[r] = val[b][2][r0 + r][lane]; rh[r] = val[b][3][r0 + r][lane];
+                }
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    if (r0 + r >= rows) break;
+                    if (k > 0 || r0 + r > 0) {
+                        const T wgt = div_by(lo[r], rec_prev);
+                        di[r] = fma_rn(-wgt, up_prev, di[r]);
+                        rh[r] = fma_rn(-wgt, rhs_prev, rh[r]);
+                    }
+                    up_prev = up[r];
+                    rec_prev = recip_relax(di[r]);
+                    rhs_prev = rh[r];
+                    if (on) {
+                        const size_t o = (size_t)(k * kGR + r0 + r) * p + c;
+                        stc(dg, o, lim, kDbgOther, rec_prev);
+                        stc(rg, o, lim, kDbgOther, rhs_prev);
+                    }
+                }
+            }
+        }
+        __syncthreads();
     }
-    T x = div_relax(crh_prev, cdi_prev);
-    stc(L.u, (size_t)(n - 1) * p + j, (size_t)n * p, kDbgOther, x);
-    for (int i1 = n - 2; i1 >= 0; i1 -= R) {
-        T gg[R + 1], d[R], rr[R];
+    // ---- substitution, upwards: chunk k from its last row
+    auto fetch = [&](int k, int b) {
+        for (int r = warp - 1; r < kGR; r += kGW - 1) {
+            const int i = k * kGR + r;
+            if (i >= n) break;
+            const size_t o = (size_t)i * p + jc, q = (size_t)i * p + (on ? c : 0);
+            const bool hS = i + 1 < n;
+            val[b][0][r][lane] = hS ? mul_rn(L.cdiff, face(__ldg(L.G + o), __ldg(L.G + o + p), true)) : T(0);
+            val[b][1][r][lane] = dg[q];
+            val[b][2][r][lane] = rg[q];
+        }
+    };
+    if (warp > 0) fetch(chunks - 1, (chunks - 1) & 1);
+    __syncthreads();
+    T x = T(0);
+    for (int k = chunks - 1; k >= 0; --k) {
+        const int b = k & 1, rows = min(kGR, n - k * kGR);
+        if (warp > 0) {
+            if (k > 0) fetch(k - 1, b ^ 1);
+        } else {
+            for (int r1 = rows - 1; r1 >= 0; r1 -= 8) {
+                T up[8], rec[8], rh[8];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int i = i1 - r;
-            if (i >= 0) {
-                const size_t o = (size_t)i * p + j;
-                gg[r] = __ldg(G + o);
-                d[r] = dg[o];
-                rr[r] = rg[o];
+                for (int r = 0; r < 8; ++r) {
+                    const int q = max(r1 - r, 0);
+                    up[r] = val[b][0][q][lane]; rec[r] = val[b][1][q][lane]; rh[r] = val[b][2][q][lane];
+                }
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    if (r1 - r < 0) break;
+                    const int i = k * kGR + r1 - r;
+                    x = i == n - 1 ? div_by(rh[r], rec[r]) : div_by(fma_rn(-up[r], x, rh[r]), rec[r]);
+                    if (on) stc(L.u, (size_t)i * p + j, lim, kDbgOther, x);
+                }
             }
         }
-        gg[R] = T(0);
-        T g_below = __ldg(G + (size_t)(i1 + 1) * p + j);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int i = i1 - r;
-            if (i < 0) break;
-            const T up = mul_rn(L.cdiff, face(gg[r], g_below, true));
-            x = div_relax(fma_rn(-up, x, rr[r]), d[r]);
-            stc(L.u, (size_t)i * p + j, (size_t)n * p, kDbgOther, x);
-            g_below = gg[r];
-        }
+        __syncthreads();
     }
 }
 
@@ -181,7 +217,7 @@ void launch_gsline(const LevelView<T> &L, cudaStream_t st) {
     for (int par = 0; par < 2; ++par) {
         const int cols = (L.m - par + 1) / 2;
         if (cols <= 0) continue;
-        k_gsline<T><<<(cols + 127) / 128, 128, 0, st>>>(L, par, L.r, L.t);
+        k_gsline<T><<<(cols + 31) / 32, 32 * kGW, 0, st>>>(L, par, L.r, L.t);
     }
 }
 
