@@ -227,7 +227,7 @@ struct Solver final : SolverBase {
     int steps = 0, cycles_step = 0, cycles_total = 0;
     int rejected = 0;             // step attempts rejected by the step control
     double tau0 = 1.0;            // tau of the parameters (the step control halves p.tau)
-    long long graph_epoch = 0;    // counts drop_graphs(): a batch rebuilds its graph when it changed
+    long long graph_epoch = 0;    // counts drop_graphs(): a batch rebuilds its graph when it changed (or tau)
     long long wait_limit = kDefaultWaitLimit;   // try_wait rounds of the TMA sweep's bounded waits
     int inject_cycle = 0;         // mg_inject_divergence: V-cycle (of a step attempt) that reports
                                   // a diverged residual once; 0 = none
@@ -276,13 +276,65 @@ struct Solver final : SolverBase {
 
     ~Solver() override { release(); }
 
+    // The graphs hold 1 / tau.  The step control tries the same few values (tau, tau / 2, ...) for
+    // image after image, and a capture with its instantiation takes 0.3 to 0.4 ms (a 256^2 step
+    // 4 ms): the graphs of the last kKeptTaus values stay with the handle.
+    struct TauGraphs {
+        double tau = 0;
+        cudaGraphExec_t gexec = nullptr, gexec_l = nullptr, gexec_li = nullptr, gloop = nullptr;
+        double gloop_tol = -1.0;
+        int gloop_max = -1;
+        bool gloop_fused = false;
+        long long gloop_nodes = 0, gloop_first = 0, graph_nodes = 0, nodes_l = 0, nodes_li = 0;
+        void destroy() {
+            for (cudaGraphExec_t *g : {&gexec, &gexec_l, &gexec_li, &gloop}) {
+                if (*g) cudaGraphExecDestroy(*g);
+                *g = nullptr;
+            }
+        }
+    };
+    static constexpr size_t kKeptTaus = 6;
+    std::vector<TauGraphs> kept;   // of other values than p.tau, the latest last
+
+    TauGraphs current_graphs() const {
+        return {p.tau, gexec, gexec_l, gexec_li, gloop, gloop_tol, gloop_max, gloop_fused, gloop_nodes, gloop_first,
+                graph_nodes, nodes_l, nodes_li};
+    }
+    void set_graphs(const TauGraphs &t) {
+        gexec = t.gexec; gexec_l = t.gexec_l; gexec_li = t.gexec_li; gloop = t.gloop;
+        gloop_tol = t.gloop_tol; gloop_max = t.gloop_max; gloop_fused = t.gloop_fused;
+        gloop_nodes = t.gloop_nodes; gloop_first = t.gloop_first;
+        graph_nodes = t.graph_nodes; nodes_l = t.nodes_l; nodes_li = t.nodes_li;
+    }
+
+    // p.tau = tau, with the graphs captured for it if they are still kept (no graph is running here:
+    // every launch is waited for).
+    void switch_tau(double tau) {
+        if (tau == p.tau) return;
+        TauGraphs next;
+        for (size_t k = 0; k < kept.size(); ++k)
+            if (kept[k].tau == tau) {
+                next = kept[k];
+                kept.erase(kept.begin() + k);
+                break;
+            }
+        kept.push_back(current_graphs());
+        if (kept.size() >= kKeptTaus) {
+            kept.front().destroy();
+            kept.erase(kept.begin());
+        }
+        set_graphs(next);
+        p.tau = tau;
+    }
+
+    // Drops the captured graphs (their kernels, shapes or launch arguments other than tau change).
     void drop_graphs() {
         ++graph_epoch;
-        if (gexec) cudaGraphExecDestroy(gexec);
-        if (gexec_l) cudaGraphExecDestroy(gexec_l);
-        if (gexec_li) cudaGraphExecDestroy(gexec_li);
-        if (gloop) cudaGraphExecDestroy(gloop);
-        gexec = gexec_l = gexec_li = gloop = nullptr;
+        TauGraphs t = current_graphs();
+        t.destroy();
+        set_graphs(TauGraphs{});
+        for (TauGraphs &g : kept) g.destroy();
+        kept.clear();
     }
 
     void release() {
@@ -575,11 +627,8 @@ struct Solver final : SolverBase {
     int reset(const void *image, const double *mk, int k) override {
         if (k > kcap) return fail(MG_ERR_ARG, "more markers than at set-up");
         // the kernels read the initial contour's area from the device scalars, so the captured
-        // graphs stay valid; only a tau changed by the step control is restored (and they go)
-        if (p.tau != tau0) {
-            p.tau = tau0;
-            drop_graphs();
-        }
+        // graphs stay valid; a tau changed by the step control is restored
+        switch_tau(tau0);
         in_step = false;
         rejected = 0;
         steps = cycles_step = cycles_total = 0;
@@ -1423,14 +1472,13 @@ struct Solver final : SolverBase {
 
     // Rejects the current attempt at a step: phi = phi^n again (the increment u of the finest
     // grid is zeroed; the coarse grids are rebuilt by every V-cycle) and the following attempts
-    // and steps use `tau` (the graphs, which hold 1/tau, are captured again).
+    // and steps use `tau` (see switch_tau).
     int restart_step(double tau) override {
         if (!in_step) return fail(MG_ERR_STATE, "restart outside a step");
         Level<T> &F = lv[0];
         CK(cudaMemset2DAsync(F.u, (size_t)F.pitch * sizeof(T), 0, (size_t)F.m * sizeof(T), F.n, st));
-        p.tau = tau;
+        switch_tau(tau);
         ++rejected;
-        drop_graphs();
         in_step = false;
         return MG_OK;
     }
@@ -1823,14 +1871,17 @@ struct Batch {
     bool own_stream = false;
     Scalars **d_sc = nullptr;
     double *d_out = nullptr, *h_out = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    cudaGraphExec_t exec = nullptr;   // every image's V-cycle
+    cudaGraphExec_t round = nullptr;  // a restart round: the V-cycles of the images that restart
     double tol_baked = -1.0;
-    std::vector<long long> epochs;   // each image's graph_epoch when the batch graph was built
+    std::vector<long long> epochs;   // each image's graph_epoch and tau when exec was built
+    std::vector<double> taus;
     int tuned_shape = -2;            // mg_batch_autotune: -1 per-image shapes, 0..5 one shape, -2 not run
 
     ~Batch() {
         if (st) cudaStreamSynchronize(st);
         if (exec) cudaGraphExecDestroy(exec);
+        if (round) cudaGraphExecDestroy(round);
         for (auto *x : s) delete x;
         for (auto *x : h) delete x;
         if (d_sc) cudaFree(d_sc);
@@ -1839,16 +1890,19 @@ struct Batch {
         if (own_stream && st) cudaStreamDestroy(st);
     }
 
-    int build(double tol) {
-        if (exec) { cudaGraphExecDestroy(exec); exec = nullptr; }
+    // The graph of one V-cycle of every image into exec, or of the images in `only` into round.
+    int build(double tol, const std::vector<char> *only = nullptr) {
+        cudaGraphExec_t &to = only ? round : exec;
+        if (to) { cudaGraphExecDestroy(to); to = nullptr; }
         const int count = (int)s.size();
         cudaGraph_t B;
         CK(cudaGraphCreate(&B, 0));
         std::vector<cudaGraphNode_t> ends;
-        nodes.assign(count, 0);
+        nodes.resize(count, 0);
         int rc = MG_OK;
         double tol2 = tol * tol;
         for (int i = 0; i < count && rc == MG_OK; ++i) {
+            if (only && !(*only)[i]) continue;
             cudaGraph_t gi;
             if ((rc = s[i]->capture_vcycle(&gi, &nodes[i]))) break;
             cudaGraphConditionalHandle hc;
@@ -1889,14 +1943,18 @@ struct Batch {
             cudaError_t e = cudaGraphAddKernelNode(&gn, B, ends.data(), ends.size(), &kp);
             if (e == cudaSuccess)
                 e = cudaGraphAddMemcpyNode1D(&mn, B, &gn, 1, h_out, d_out, sizeof(double) * 3 * count, cudaMemcpyDeviceToHost);
-            if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, B, 0);
-            if (e != cudaSuccess) { exec = nullptr; rc = fail(MG_ERR_CUDA, std::string("batch graph: ") + cudaGetErrorString(e)); }
+            if (e == cudaSuccess) e = cudaGraphInstantiate(&to, B, 0);
+            if (e != cudaSuccess) { to = nullptr; rc = fail(MG_ERR_CUDA, std::string("batch graph: ") + cudaGetErrorString(e)); }
         }
         cudaGraphDestroy(B);
-        if (rc == MG_OK) {
+        if (rc == MG_OK && !only) {
             tol_baked = tol;
             epochs.resize(count);
-            for (int i = 0; i < count; ++i) epochs[i] = s[i]->graph_epoch;
+            taus.resize(count);
+            for (int i = 0; i < count; ++i) {
+                epochs[i] = s[i]->graph_epoch;
+                taus[i] = s[i]->p.tau;
+            }
         }
         return rc;
     }
@@ -1956,7 +2014,7 @@ struct Batch {
     // that has not reached tol.  The step control of mg_solve_step applies per image, in rounds:
     // an image whose attempt stalls, diverges or reaches max_cycles V-cycles is halted on the
     // device; once no image is left running, the halted ones restart from their phi^n with
-    // tau / 2 together (one rebuild of the batch graph per round).
+    // tau / 2 together, as a graph of their V-cycles alone.
     int solve_step(double tol, int max_cycles, int *cycles, double *rho) {
         const int count = (int)s.size();
         for (int i = 0; i < count; ++i) {
@@ -1964,7 +2022,7 @@ struct Batch {
             if (rc) return rc;
         }
         bool stale = !exec || tol != tol_baked || (int)epochs.size() != count;
-        for (int i = 0; i < count && !stale; ++i) stale = s[i]->graph_epoch != epochs[i];
+        for (int i = 0; i < count && !stale; ++i) stale = s[i]->graph_epoch != epochs[i] || s[i]->p.tau != taus[i];
         if (stale) {
             int rc = build(tol);
             if (rc) return rc;
@@ -1974,10 +2032,11 @@ struct Batch {
         std::vector<std::vector<double>> hist(count);
         std::vector<char> active(count, 1), failed(count, 0), restart(count, 0);
         int rc = MG_OK;
+        cudaGraphExec_t cur = exec;
         for (;;) {
             bool any = true;
             while (any && rc == MG_OK) {
-                CK(cudaGraphLaunch(exec, st));
+                CK(cudaGraphLaunch(cur, st));
                 CK(cudaStreamSynchronize(st));
                 any = false;
                 for (int i = 0; i < count; ++i) {
@@ -2030,7 +2089,8 @@ struct Batch {
                 again = true;
             }
             if (rc || !again) break;
-            if ((rc = build(tol))) break;
+            if ((rc = build(tol, &active))) break;   // the others are done
+            cur = round;
         }
         if (cycles) for (int i = 0; i < count; ++i) cycles[i] = cyc[i];
         if (rho) for (int i = 0; i < count; ++i) rho[i] = r[i];
