@@ -86,6 +86,53 @@ __global__ void __launch_bounds__(256, MINB)
     }
 }
 
+// The same residual without the norm on tiles of H x 32 cells: FP64 grids that leave SMs idle with
+// square tiles (an SM's FP64 units are the bound; see thin tiles in smooth_kernels.cu).
+template <typename T, int H>
+__global__ void __launch_bounds__(32 * H) k_residual_thin(LevelView<T> L, const T *uin, const double *area, T *out, int mode) {
+    constexpr int NT = 32 * H;
+    __shared__ T sP[H + 4][37], sU[H + 4][37], sG[H + 2][35];
+    const int i0 = blockIdx.y * H, j0 = blockIdx.x * 32;
+    const int lane = threadIdx.x, wy = threadIdx.y, tid = wy * 32 + lane;
+    const int n = L.n, m = L.m, p = L.pitch;
+    const size_t lim = (size_t)n * p;
+    pdl_wait();
+    pdl_trigger();
+    for (int q = tid; q < (H + 4) * 36; q += NT) {
+        const int a = q / 36, b = q - a * 36;
+        const size_t o = (size_t)clamp_idx(i0 - 2 + a, n - 1) * p + clamp_idx(j0 - 2 + b, m - 1);
+        sP[a][b] = ldl2(L.pn, o, lim, kDbgResidual);
+        sU[a][b] = ldl2(uin, o, lim, kDbgResidual);
+    }
+    __syncthreads();
+    for (int q = tid; q < (H + 2) * 34; q += NT) {
+        const int a = q / 34, b = q - a * 34, gi = i0 - 1 + a, gj = j0 - 1 + b;
+        T g = T(0);
+        if (gi >= 0 && gi < n && gj >= 0 && gj < m)
+            g = cell_G(weight_at(L, (size_t)gi * p + gj), sP[a + 2][b + 1], sP[a][b + 1], sP[a + 1][b + 2], sP[a + 1][b],
+                       sU[a + 2][b + 1], sU[a][b + 1], sU[a + 1][b + 2], sU[a + 1][b], L.inv_2h, L.beta);
+        sG[a][b] = g;
+    }
+    __syncthreads();
+    const int gi = i0 + wy, gj = j0 + lane, a = wy + 2, b = lane + 2;
+    const size_t o = (size_t)gi * p + gj;
+    if (gi >= n || gj >= m || !MG_DBG_OK(o, lim, kDbgResidual)) return;
+    const bool hS = gi + 1 < n, hN = gi > 0, hE = gj + 1 < m, hW = gj > 0;
+    const T gc = sG[wy + 1][lane + 1];
+    // doubled faces, with cdiff / 2 (face2 in arith.cuh: the same values)
+    const T aS = face2(gc, sG[wy + 2][lane + 1], hS), aN = face2(gc, sG[wy][lane + 1], hN);
+    const T aE = face2(gc, sG[wy + 1][lane + 2], hE), aW = face2(gc, sG[wy + 1][lane], hW);
+    const T pc = sP[a][b], uc = sU[a][b];
+    T fl = mul_rn(aS, add_rn(sub_rn(sP[a + 1][b], pc), sub_rn(sU[a + 1][b], uc)));
+    fl = fma_rn(aN, add_rn(sub_rn(sP[a - 1][b], pc), sub_rn(sU[a - 1][b], uc)), fl);
+    fl = fma_rn(aE, add_rn(sub_rn(sP[a][b + 1], pc), sub_rn(sU[a][b + 1], uc)), fl);
+    fl = fma_rn(aW, add_rn(sub_rn(sP[a][b - 1], pc), sub_rn(sU[a][b - 1], uc)), fl);
+    const T ar = area ? T(__ldcg(area + L.level)) : T(0);
+    const T Lv = sub_rn(fma_rn(L.cdiff * T(0.5), fl, -add_rn(__ldcg(L.F + o), ar)), mul_rn(L.inv_tau, uc));
+    if (mode == 0) out[o] = L.has_rhs ? sub_rn(__ldcg(L.rhs + o), Lv) : -Lv;
+    else out[o] = add_rn(__ldcg(out + o), Lv);
+}
+
 // Loads the window dst[a][b] = src[clamp(r0 + a)][clamp(c0 + b)], a < ROWS, b < COLS, of one or
 // two pitched FP32 grid functions (indices clamped into the grid: the mirror ghosts), with
 // 16-byte vector loads where the window lies inside; c0 mod 4 == OFF.  NT threads.
@@ -229,6 +276,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_restrict(RestrictFields<T> F, int n, int m, int pf, int pc) {
     const int J = blockIdx.x * 32 + threadIdx.x, I = blockIdx.y * 8 + threadIdx.y;
     const int nc = n / 2, mc = m / 2;
+    pdl_wait();
+    pdl_trigger();
     if (I >= nc || J >= mc) return;
     const T *f = F.f[blockIdx.z];
     T *c = F.c[blockIdx.z], *c2 = F.c2[blockIdx.z];
@@ -239,7 +288,7 @@ __global__ void __launch_bounds__(256) k_restrict(RestrictFields<T> F, int n, in
     for (int a = 0; a < nr; ++a) {
         T row = T(0);
         for (int b = 0; b < nk; ++b)
-            row = fma_rn(T(cw[b]), ldc(f, (size_t)ri[a] * pf + ci[b], (size_t)n * pf, kDbgResidual), row);
+            row = fma_rn(T(cw[b]), ldl2(f, (size_t)ri[a] * pf + ci[b], (size_t)n * pf, kDbgResidual), row);
         s = fma_rn(T(rw[a]), row, s);
     }
     stc(c, (size_t)I * pc + J, (size_t)nc * pc, kDbgResidual, s);
@@ -250,6 +299,8 @@ __global__ void __launch_bounds__(256) k_restrict(RestrictFields<T> F, int n, in
 template <typename T>
 __global__ void __launch_bounds__(256) k_interp_add(LevelView<T> Lf, LevelView<T> Lc) {
     const int j = blockIdx.x * 32 + threadIdx.x, i = blockIdx.y * 8 + threadIdx.y;
+    pdl_wait();
+    pdl_trigger();
     if (i >= Lf.n || j >= Lf.m) return;
     int ri[2], ci[2];
     float rw[2], cw[2];
@@ -258,10 +309,11 @@ __global__ void __launch_bounds__(256) k_interp_add(LevelView<T> Lf, LevelView<T
     for (int a = 0; a < nr; ++a)
         for (int b = 0; b < nk; ++b) {
             size_t o = (size_t)ri[a] * Lc.pitch + ci[b], lc = (size_t)Lc.n * Lc.pitch;
-            s = fma_rn(T(rw[a] * cw[b]), sub_rn(ldc(Lc.u, o, lc, kDbgInterp), ldc(Lc.u0, o, lc, kDbgInterp)), s);
+            s = fma_rn(T(rw[a] * cw[b]), sub_rn(ldl2(Lc.u, o, lc, kDbgInterp), ldl2(Lc.u0, o, lc, kDbgInterp)), s);
         }
     size_t o = (size_t)i * Lf.pitch + j;
-    stc(Lf.u, o, (size_t)Lf.n * Lf.pitch, kDbgInterp, add_rn(Lf.u[o], s));
+    const size_t lf = (size_t)Lf.n * Lf.pitch;
+    stc(Lf.u, o, lf, kDbgInterp, add_rn(ldl2(Lf.u, o, lf, kDbgInterp), s));
 }
 
 // The coarsest solve (coarse_body.cuh) as its own one-block kernel.
@@ -316,6 +368,13 @@ void launch_residual(const LevelView<T> &L, const T *uin, const double *area, T 
     // register-limited FP32 variant when it makes every tile resident at once (same operations,
     // same order)
     const ResOcc &o = res_occ();
+    if constexpr (sizeof(T) == 8) {
+        if (!norm_out && (long)grid.x * grid.y < o.sms) {   // square tiles leave SMs idle
+            constexpr int H = 4;
+            launch_pdl(k_residual_thin<T, H>, dim3(grid.x, (L.n + H - 1) / H), dim3(32, H), 0, st, L, uin, area, out, mode);
+            return;
+        }
+    }
     if (sizeof(T) == 4 && (long)grid.x * grid.y <= (long)o.sms * o.per_sm)
         k_residual<T, sizeof(T) == 4 ? 8 : 1><<<grid, block, 0, st>>>(L, uin, area, out, mode,
                                                                       norm_out ? partials : nullptr);
@@ -334,13 +393,13 @@ void launch_restrict(const T *f, int n, int m, int pf, T *c, T *c2, int pc, cuda
 template <typename T>
 void launch_restrict_fields(const RestrictFields<T> &F, int n, int m, int pf, int pc, cudaStream_t st) {
     dim3 grid((m / 2 + 31) / 32, (n / 2 + 7) / 8, F.nf), block(32, 8);
-    k_restrict<T><<<grid, block, 0, st>>>(F, n, m, pf, pc);
+    launch_pdl(k_restrict<T>, grid, block, 0, st, F, n, m, pf, pc);
 }
 
 template <typename T>
 void launch_interp_add(const LevelView<T> &Lf, const LevelView<T> &Lc, cudaStream_t st) {
     dim3 grid((Lf.m + 31) / 32, (Lf.n + 7) / 8), block(32, 8);
-    k_interp_add<T><<<grid, block, 0, st>>>(Lf, Lc);
+    launch_pdl(k_interp_add<T>, grid, block, 0, st, Lf, Lc);
 }
 
 constexpr size_t kCoarseSmemMax = 200 * 1024;

@@ -79,6 +79,12 @@ __device__ __forceinline__ T ldc(const T *p, size_t i, size_t lim, int site) {
 #endif
     return p[i];
 }
+
+// ... through L2: what the kernel before a dependent launch has written.
+template <typename T>
+__device__ __forceinline__ T ldl2(const T *p, size_t i, size_t lim, int site) {
+    return MG_DBG_OK(i, lim, site) ? __ldcg(p + i) : T(0);
+}
 template <typename T>
 __device__ __forceinline__ void stc(T *p, size_t i, size_t lim, int site, T v) {
 #ifdef MG_DEBUG

@@ -55,9 +55,9 @@ __device__ __forceinline__ void tile_line_phases(UA U, GA Gc, FA Fc, MA MK, int 
                     const int a = ROWWISE ? li : s0 + t, b = ROWWISE ? s0 + t : li;
                     const int gi = i0 - KH + a, gj = j0 - KH + b;
                     const bool hS = gi + 1 < n, hN = gi > 0, hE = gj + 1 < m, hW = gj > 0;
-                    const T gc = Gc(a, b);
-                    const T aS = face(gc, Gc(a + 1, b), hS), aN = face(gc, Gc(a - 1, b), hN);
-                    const T aE = face(gc, Gc(a, b + 1), hE), aW = face(gc, Gc(a, b - 1), hW);
+                    const T gc = Gc(a, b);   // doubled faces, with cdiff / 2 (face2 in arith.cuh)
+                    const T aS = face2(gc, Gc(a + 1, b), hS), aN = face2(gc, Gc(a - 1, b), hN);
+                    const T aE = face2(gc, Gc(a, b + 1), hE), aW = face2(gc, Gc(a, b - 1), hW);
                     RunCell<T> c;
                     if (ROWWISE) {
                         c.ap = aW; c.an = aE; c.ax1 = aS; c.ax2 = aN;
@@ -70,7 +70,7 @@ __device__ __forceinline__ void tile_line_phases(UA U, GA Gc, FA Fc, MA MK, int 
                     return c;
                 };
                 T x;
-                if (pcr_piece<T>(mk, len, cdiff, inv_tau, own, endp, endn, at, x)) {
+                if (pcr_piece<T>(mk, len, cdiff * T(0.5), inv_tau, own, endp, endn, at, x)) {
                     if (ROWWISE) U(li, pos) = x; else U(pos, li) = x;
                 }
             }

@@ -16,6 +16,7 @@
 //     depends on another within a sweep.
 #include "arith.cuh"
 #include "line_phase.cuh"
+#include "tma.cuh"
 
 namespace segmg {
 
@@ -144,6 +145,92 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_snapshot(LevelView<T> L, c
     }
 }
 
+// The same snapshot in FP64 on small grids: a cluster of 32 / H blocks shares a 32 x 32 tile, H rows
+// (and warps) a block, since one SM's FP64 units are the bound (35,000 cycles a tile, G's square root
+// and division most of it).  A block knows H bits of its columns' star masks; they go to the
+// cluster's first block (distributed shared memory), which finishes the column pieces.
+template <typename T, int H>
+__global__ void __launch_bounds__(32 * H) k_snapshot_thin(LevelView<T> L, const double *area) {
+    constexpr int NB = 32 / H, NT = 32 * H;   // blocks of the cluster; threads
+    __shared__ T sP[H + 4][37], sU[H + 4][37], sG[H + 2][35];
+    __shared__ uint8_t sStar[H][32];
+    __shared__ uint32_t colw[2][NB][32];   // first block: sweeps C, D, bits of each block's rows
+    const int rank = blockIdx.y % NB;
+    const int i0 = blockIdx.y * H, j0 = blockIdx.x * 32, t0 = i0 - rank * H;   // t0: the tile's first row
+    const int lane = threadIdx.x, wy = threadIdx.y, tid = wy * 32 + lane;
+    const int n = L.n, m = L.m, p = L.pitch;
+    const size_t lim = (size_t)n * p;
+    pdl_wait();
+    pdl_trigger();
+    for (int q = tid; q < (H + 4) * 36; q += NT) {   // pn, u on rows i0-2 .., mirror-clamped
+        const int a = q / 36, b = q - a * 36;
+        const size_t o = (size_t)clamp_idx(i0 - 2 + a, n - 1) * p + clamp_idx(j0 - 2 + b, m - 1);
+        sP[a][b] = ldl2(L.pn, o, lim, kDbgSnapshot);
+        sU[a][b] = ldl2(L.u, o, lim, kDbgSnapshot);
+    }
+    __syncthreads();
+    for (int q = tid; q < (H + 2) * 34; q += NT) {   // G on rows i0-1 .., columns j0-1 ..
+        const int a = q / 34, b = q - a * 34, gi = i0 - 1 + a, gj = j0 - 1 + b;
+        T g = T(0);
+        if (gi >= 0 && gi < n && gj >= 0 && gj < m)
+            g = cell_G(weight_at(L, (size_t)gi * p + gj), sP[a + 2][b + 1], sP[a][b + 1], sP[a + 1][b + 2], sP[a + 1][b],
+                       sU[a + 2][b + 1], sU[a][b + 1], sU[a + 1][b + 2], sU[a + 1][b], L.inv_2h, L.beta);
+        sG[a][b] = g;
+    }
+    __syncthreads();
+    const int gi = i0 + wy, gj = j0 + lane;
+    uint8_t star = 0;
+    if (gi < n && gj < m) {
+        const T ar = area ? T(__ldcg(area + L.level)) : T(0);
+        const bool hS = gi + 1 < n, hN = gi > 0, hE = gj + 1 < m, hW = gj > 0;
+        const T gc = sG[wy + 1][lane + 1];
+        // doubled faces, with cdiff / 2 (face2 in arith.cuh: the same values)
+        const T aS = face2(gc, sG[wy + 2][lane + 1], hS), aN = face2(gc, sG[wy][lane + 1], hN);
+        const T aE = face2(gc, sG[wy + 1][lane + 2], hE), aW = face2(gc, sG[wy + 1][lane], hW);
+        const int a = wy + 2, b = lane + 2;
+        const T pc = sP[a][b];
+        T ds = mul_rn(aS, sub_rn(sP[a + 1][b], pc));
+        ds = fma_rn(aN, sub_rn(sP[a - 1][b], pc), ds);
+        ds = fma_rn(aE, sub_rn(sP[a][b + 1], pc), ds);
+        ds = fma_rn(aW, sub_rn(sP[a][b - 1], pc), ds);
+        const size_t o = (size_t)gi * p + gj;
+        T base = add_rn(ldl2(L.F, o, lim, kDbgSnapshot), ar);
+        if (L.has_rhs) base = add_rn(base, ldl2(L.rhs, o, lim, kDbgSnapshot));
+        stc(L.f, o, lim, kDbgSnapshot, fma_rn(-(L.cdiff * T(0.5)), ds, base));
+        stc(L.G, o, lim, kDbgSnapshot, gc);
+        const T big = T(3.0e38);
+        const T vS = hS ? aS : big, vN = hN ? aN : big, vE = hE ? aE : big, vW = hW ? aW : big;
+        const T mn = fmin(fmin(vS, vN), fmin(vE, vW));
+        const T mx = fmax(fmax(hS ? aS : T(-1), hN ? aN : T(-1)), fmax(hE ? aE : T(-1), hW ? aW : T(-1)));
+        const int am = vS == mn ? 0 : (vN == mn ? 1 : (vE == mn ? 2 : 3));
+        const int cnt = (int)hS + (int)hN + (int)hE + (int)hW;
+        if (cnt >= 2 && mx > mul_rn(L.Sigma, mn)) star = (uint8_t)(1u << am);
+        if (L.cls) stc(L.cls, o, lim, kDbgSnapshot, star);
+    }
+    sStar[wy][lane] = star;
+    const uint32_t bA = __ballot_sync(0xffffffffu, star & 1u), bB = __ballot_sync(0xffffffffu, star & 2u);
+    if (lane < 2 && gi < n)
+        stc(L.mrow, ((size_t)lane * n + gi) * L.npm + (j0 >> 5), (size_t)2 * n * L.npm, kDbgMaskStore,
+            members_of(lane ? bB : bA, min(32, m - j0)));
+    __syncthreads();
+    if (wy < 2) {   // warp 0: sweep C, warp 1: sweep D
+        uint32_t v = 0;
+#pragma unroll
+        for (int r = 0; r < H; ++r) v |= ((sStar[r][lane] >> (2 + wy)) & 1u) << (rank * H + r);
+        uint32_t at;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;\n" : "=r"(at) : "r"(smem_u32(&colw[wy][rank][lane])));
+        asm volatile("st.shared::cluster.u32 [%0], %1;\n" ::"r"(at), "r"(v) : "memory");
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    if (rank == 0 && wy < 2 && gj < m) {
+        uint32_t v = 0;
+#pragma unroll
+        for (int r = 0; r < NB; ++r) v |= colw[wy][r][lane];
+        stc(L.mcol, ((size_t)wy * m + gj) * L.npn + (t0 >> 5), (size_t)2 * m * L.npn, kDbgMaskStore,
+            members_of(v, min(32, n - t0)));
+    }
+}
+
 // ---------------------------------------------------------------------------------------
 // Phased path
 // ---------------------------------------------------------------------------------------
@@ -234,6 +321,14 @@ using Tile2 = TileShape<64, 64, 512>;
 using Tile3 = TileShape<32, 64, 512>;   // more threads per tile: fewer cells per thread per phase
 using Tile4 = TileShape<32, 32, 256>;
 using Tile5 = TileShape<32, 32, 512>;   // one cell per thread per checkerboard phase
+// FP64: thin tiles of H rows (row sweeps) or H columns (column sweeps).  An SM has two FP64
+// multiply-adds a cycle, so a sweep's time is the cells of the busiest SM: on grids below about 400^2
+// the square tiles leave SMs idle (128^2: 16 of 152 busy, 26 us a sweep), and thin ones spread the
+// work, halo included, over all of them (see thin_rows).
+template <int H>
+using ThinRows = TileShape<H, 32, 128>;
+template <int H>
+using ThinCols = TileShape<32, H, 128>;
 
 template <typename T, typename TS>
 struct FusedSmem {
@@ -273,9 +368,9 @@ __device__ __forceinline__ void rb_phase(FusedSmem<T, TS> &S, const LevelView<T>
         }
         if (tile_member<T, TS, (SWEEP < 2)>(S, a, b)) continue;
         const T gc = S.G[colour][a][k];
-        const T aS = face(gc, S.G[other][a + 1][k], hS), aN = face(gc, S.G[other][a - 1][k], hN);
-        const T aE = face(gc, S.G[other][a][k + x], hE), aW = face(gc, S.G[other][a][k + x - 1], hW);
-        T v = point_relax(L.cdiff, L.inv_tau, aS, aN, aE, aW, S.u[other][a + 1][k], S.u[other][a - 1][k],
+        const T aS = face2(gc, S.G[other][a + 1][k], hS), aN = face2(gc, S.G[other][a - 1][k], hN);
+        const T aE = face2(gc, S.G[other][a][k + x], hE), aW = face2(gc, S.G[other][a][k + x - 1], hW);
+        T v = point_relax(L.cdiff * T(0.5), L.inv_tau, aS, aN, aE, aW, S.u[other][a + 1][k], S.u[other][a - 1][k],
                           S.u[other][a][k + x], S.u[other][a][k + x - 1], S.f[colour][a][k]);
         if (WEIGHTED) {
             const size_t o = (size_t)(i0 - kH + a) * L.pitch + (j0 - kH + b);
@@ -301,6 +396,8 @@ __global__ void __launch_bounds__(TS::NT) k_sweep(LevelView<T> L) {
     // no tile can read a neighbour's already updated cells
     const T *uin = (SWEEP & 1) ? L.t : L.u;
     T *uout = (SWEEP & 1) ? L.u : L.t;
+    pdl_wait();
+    pdl_trigger();
     // ---- load u, G, f as vectors (the region starts 16-byte aligned): all loads of a batch are
     // issued before any shared-memory store, so they are in flight together
     constexpr int NVEC = kRH * NV, PER = (NVEC + kThreads - 1) / kThreads, BATCH = VN == 4 ? PER : 3;
@@ -315,9 +412,9 @@ __global__ void __launch_bounds__(TS::NT) k_sweep(LevelView<T> L) {
             if (k0 + k < PER && q < NVEC && gi >= 0 && gi < n && gj >= 0 && gj < p &&
                 MG_DBG_OK((size_t)gi * p + gj + VN - 1, (size_t)n * p, kDbgSweep)) {
                 const size_t o = (size_t)gi * p + gj;
-                x[k][0] = __ldg(reinterpret_cast<const V *>(uin + o));
-                x[k][1] = __ldg(reinterpret_cast<const V *>(L.G + o));
-                x[k][2] = __ldg(reinterpret_cast<const V *>(L.f + o));
+                x[k][0] = __ldcg(reinterpret_cast<const V *>(uin + o));
+                x[k][1] = __ldcg(reinterpret_cast<const V *>(L.G + o));
+                x[k][2] = __ldcg(reinterpret_cast<const V *>(L.f + o));
             } else {
                 memset(&x[k][0], 0, 3 * sizeof(V));
             }
@@ -346,7 +443,7 @@ __global__ void __launch_bounds__(TS::NT) k_sweep(LevelView<T> L) {
             uint32_t w = 0;
             if (gi >= 0 && gi < n && piece >= 0 && piece < L.npm &&
                 MG_DBG_OK(((size_t)SWEEP * n + gi) * L.npm + piece, (size_t)2 * n * L.npm, kDbgMaskLoad))
-                w = __ldg(L.mrow + ((size_t)SWEEP * n + gi) * L.npm + piece);
+                w = __ldcg(L.mrow + ((size_t)SWEEP * n + gi) * L.npm + piece);
             S.mk[a][pc] = w;
             lm |= solves_word<kH, kOH, kOW, true>(a, pc, w);
         }
@@ -357,7 +454,7 @@ __global__ void __launch_bounds__(TS::NT) k_sweep(LevelView<T> L) {
             uint32_t w = 0;
             if (gj >= 0 && gj < m && piece >= 0 && piece < L.npn &&
                 MG_DBG_OK(((size_t)(SWEEP - 2) * m + gj) * L.npn + piece, (size_t)2 * m * L.npn, kDbgMaskLoad))
-                w = __ldg(L.mcol + ((size_t)(SWEEP - 2) * m + gj) * L.npn + piece);
+                w = __ldcg(L.mcol + ((size_t)(SWEEP - 2) * m + gj) * L.npn + piece);
             S.mk[b][pc] = w;
             lm |= solves_word<kH, kOH, kOW, false>(b, pc, w);
         }
@@ -424,12 +521,37 @@ const SnapOcc<T> &snap_occ() {
     return o;
 }
 
+template <int H>
+static void launch_snapshot_thin(const LevelView<double> &L, const double *area, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((L.m + 31) / 32, (L.n + 31) / 32 * (32 / H));
+    cfg.blockDim = dim3(32, H);
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1;
+    at[0].val.clusterDim.y = 32 / H;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    cudaLaunchKernelEx(&cfg, k_snapshot_thin<double, H>, L, area);
+}
+
 // The most threads per tile with which every tile of the grid still gets a resident block.
 template <typename T>
 void launch_snapshot(const LevelView<T> &L, const double *area, cudaStream_t st) {
     dim3 grid((L.m + 31) / 32, (L.n + 31) / 32);
     const long tiles = (long)grid.x * grid.y;
     const SnapOcc<T> &o = snap_occ<T>();
+    if constexpr (sizeof(T) == 8) {
+        // the busiest SM's G cells (about 40 FP64 operations each) and f cells (30): a tile, or its
+        // 4- or 8-row parts
+        auto cost = [&](int h) { return (tiles * (32 / h) + o.sms - 1) / o.sms * ((h + 2) * 34 * 40 + h * 32 * 30); };
+        if (cost(4) < cost(8) && cost(4) < cost(32)) return launch_snapshot_thin<4>(L, area, st);
+        if (cost(8) < cost(32)) return launch_snapshot_thin<8>(L, area, st);
+    }
     if (tiles <= (long)o.sms * o.per_sm[2])
         k_snapshot<T, 32><<<grid, dim3(32, 32), 0, st>>>(L, area);
     else if (tiles <= (long)o.sms * o.per_sm[1])
@@ -478,6 +600,8 @@ void prepare_smoother_kernels() {
     set_fused_attrs<float, Tile3>(); set_fused_attrs<float, Tile4>(); set_fused_attrs<float, Tile5>();
     set_fused_attrs<double, Tile0>(); set_fused_attrs<double, Tile1>(); set_fused_attrs<double, Tile2>();
     set_fused_attrs<double, Tile3>(); set_fused_attrs<double, Tile4>(); set_fused_attrs<double, Tile5>();
+    set_fused_attr<double, 0, ThinRows<8>>(); set_fused_attr<double, 1, ThinRows<8>>();
+    set_fused_attr<double, 2, ThinCols<8>>(); set_fused_attr<double, 3, ThinCols<8>>();
     (void)snap_occ<double>();   // snapshot occupancy, measured here rather than inside a capture
 }
 
@@ -485,7 +609,7 @@ template <typename T, int SW, typename TS>
 static void launch_fused_one(const LevelView<T> &L, cudaStream_t st) {
     size_t smem = sizeof(FusedSmem<T, TS>);
     dim3 grid((L.m + TS::OW - 1) / TS::OW, (L.n + TS::OH - 1) / TS::OH);
-    k_sweep<T, SW, TS><<<grid, TS::NT, smem, st>>>(L);
+    launch_pdl(k_sweep<T, SW, TS>, grid, dim3(TS::NT), smem, st, L);
 }
 
 template <typename T, typename TS>
@@ -498,8 +622,41 @@ static void launch_fused_shape(const LevelView<T> &L, int sweep, cudaStream_t st
     }
 }
 
+// Rows (or columns) of a thin FP64 tile with which the busiest SM has the fewest cells to update: the
+// blocks an SM gets times the cells of a tile's two checkerboard phases (32: the square tile).
+static int thin_size(long across, long pieces, int sms) {
+    int best = 32;
+    long least = -1;
+    for (int h : {32, 8, 4, 2}) {
+        const long blocks = (across + h - 1) / h * pieces;
+        const long cost = (blocks + sms - 1) / sms * ((h + 6) * 38 + (h + 4) * 36);
+        if (least < 0 || cost < least) {
+            least = cost;
+            best = h;
+        }
+    }
+    return best;
+}
+
+template <int H>
+static void launch_thin(const LevelView<double> &L, int sweep, cudaStream_t st) {
+    switch (sweep) {
+        case 0: launch_fused_one<double, 0, ThinRows<H>>(L, st); break;
+        case 1: launch_fused_one<double, 1, ThinRows<H>>(L, st); break;
+        case 2: launch_fused_one<double, 2, ThinCols<H>>(L, st); break;
+        default: launch_fused_one<double, 3, ThinCols<H>>(L, st); break;
+    }
+}
+
 template <typename T>
 void launch_sweep_fused(const LevelView<T> &L, int sweep, int shape, cudaStream_t st) {
+    if constexpr (sizeof(T) == 8) {   // the square 32-cell shapes
+        const long rp = (L.m + 31) / 32, cp = (L.n + 31) / 32;
+        const int h = shape < 4 ? 32 : (sweep < 2 ? thin_size(L.n, rp, snap_occ<T>().sms) : thin_size(L.m, cp, snap_occ<T>().sms));
+        if (h == 8) return launch_thin<8>(L, sweep, st);
+        if (h == 4) return launch_thin<4>(L, sweep, st);
+        if (h == 2) return launch_thin<2>(L, sweep, st);
+    }
     if (shape == 1) launch_fused_shape<T, Tile1>(L, sweep, st);
     else if (shape == 2) launch_fused_shape<T, Tile2>(L, sweep, st);
     else if (shape == 3) launch_fused_shape<T, Tile3>(L, sweep, st);

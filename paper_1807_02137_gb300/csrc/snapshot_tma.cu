@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(32 * WARPS, MINB)
             float e = 0.f;
             if (I < Cg.n && J < Cg.m) {
                 const size_t o = (size_t)I * Cg.pitch + J;
-                if (MG_DBG_OK(o, lc, kDbgInterp)) e = sub_rn(__ldcg(Cg.u + o), __ldcg(Cg.u0 + o));
+                e = sub_rn(ldl2(Cg.u, o, lc, kDbgInterp), ldl2(Cg.u0, o, lc, kDbgInterp));
             }
             S.E[r][cc] = e;
         }
