@@ -160,6 +160,8 @@ __global__ void __launch_bounds__(32 * H) k_snapshot_thin(LevelView<T> L, const 
     const int lane = threadIdx.x, wy = threadIdx.y, tid = wy * 32 + lane;
     const int n = L.n, m = L.m, p = L.pitch;
     const size_t lim = (size_t)n * p;
+    // the first block's shared memory may be written once that block runs: waited for before the stores
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
     pdl_wait();
     pdl_trigger();
     for (int q = tid; q < (H + 4) * 36; q += NT) {   // pn, u on rows i0-2 .., mirror-clamped
@@ -213,6 +215,7 @@ __global__ void __launch_bounds__(32 * H) k_snapshot_thin(LevelView<T> L, const 
         stc(L.mrow, ((size_t)lane * n + gi) * L.npm + (j0 >> 5), (size_t)2 * n * L.npm, kDbgMaskStore,
             members_of(lane ? bB : bA, min(32, m - j0)));
     __syncthreads();
+    asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory");
     if (wy < 2) {   // warp 0: sweep C, warp 1: sweep D
         uint32_t v = 0;
 #pragma unroll
