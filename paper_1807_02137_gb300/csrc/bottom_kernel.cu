@@ -472,8 +472,19 @@ __device__ __forceinline__ void tile_smooth(const TileArgs &A, TileScratch &S, C
         own_push = push_of(*T, w, lane, i0, j0, n, m, rank, TX);
         line_push = push_of(*T, lane, w, i0, j0, n, m, rank, TX);
     }
-    // G at pn + u of the own cell
+    // G at pn + u of the own cell; fas: the differences of pn + u to the neighbours too, since after the
+    // next barrier a neighbouring tile may be at its first checkerboard phase, whose pushes change this
+    // tile's ring of u
+    float uc = 0.f, dS = 0.f, dN = 0.f, dE = 0.f, dW = 0.f;
     {
+        if (fas) {
+            const float pc = P[o];
+            uc = U[o];
+            dS = add_rn(sub_rn(P[oS], pc), sub_rn(U[oS], uc));
+            dN = add_rn(sub_rn(P[oN], pc), sub_rn(U[oN], uc));
+            dE = add_rn(sub_rn(P[oE], pc), sub_rn(U[oE], uc));
+            dW = add_rn(sub_rn(P[oW], pc), sub_rn(U[oW], uc));
+        }
         const float g = cell_G(smf[A.W + oc], P[oS], P[oN], P[oE], P[oW], U[oS], U[oN], U[oE], U[oW], A.inv_2h, A.beta);
         if (own) {
             G[o] = g;
@@ -495,11 +506,10 @@ __device__ __forceinline__ void tile_smooth(const TileArgs &A, TileScratch &S, C
         ds = fma_rn(aW, sub_rn(pW, pc), ds);
         float base = add_rn(smf[A.F + oc], 0.0f);
         if (fas) {   // as b_residual, mode 1, with uu = u (= u0 here)
-            const float uc = U[o];
-            float fl = mul_rn(aS, add_rn(sub_rn(pS, pc), sub_rn(U[oS], uc)));
-            fl = fma_rn(aN, add_rn(sub_rn(pN, pc), sub_rn(U[oN], uc)), fl);
-            fl = fma_rn(aE, add_rn(sub_rn(pE, pc), sub_rn(U[oE], uc)), fl);
-            fl = fma_rn(aW, add_rn(sub_rn(pW, pc), sub_rn(U[oW], uc)), fl);
+            float fl = mul_rn(aS, dS);
+            fl = fma_rn(aN, dN, fl);
+            fl = fma_rn(aE, dE, fl);
+            fl = fma_rn(aW, dW, fl);
             const float rn = add_rn(smf[A.R + oc], sub_rn(fma_rn(cdiff, fl, -base), mul_rn(inv_tau, uc)));
             if (own) smf[A.R + oc] = rn;
             base = add_rn(base, rn);
