@@ -31,15 +31,17 @@ namespace {
 // runs the 32 recurrences from values in shared memory, and the block's other warps form those
 // values (faces, products, right-hand sides) and store the results, a chunk of kGR rows ahead and
 // behind.  (One thread a column that also loaded and formed its values took about 250 cycles a row
-// each way: 4.2 ms a V-cycle at 1024^2.)
+// each way: 4.2 ms a V-cycle at 1024^2.)  A forming warp takes neighbouring rows with all their loads
+// in flight: 1024^2 step 40.4 -> 39.7 ms against one row at a time; the chain is what is left.
 // dg / rg: scratch for what the eliminated rows leave (the reciprocal of the diagonal, or in FP64 the
 // diagonal, and the right-hand side), row by row at the columns' own order (pitched like the grid).
 // ---------------------------------------------------------------------------------------
-constexpr int kGW = 8;     // warps: the solving one and seven that form values
+constexpr int kGF = 8, kGW = 1 + kGF;   // warps that form values; with the solving one
 
 template <typename T>
 __global__ void __launch_bounds__(32 * kGW) k_gsline(LevelView<T> L, int parity, T *__restrict__ dg, T *__restrict__ rg) {
     constexpr int kGR = 128 / sizeof(T);   // rows of a chunk (32 KB of values in two chunks)
+    constexpr int kFR = kGR / kGF;         // neighbouring rows of a chunk that a forming warp takes
     // down: lo, up, diagonal, right-hand side; up: up, reciprocal, right-hand side
     __shared__ T val[2][4][kGR][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -51,22 +53,35 @@ __global__ void __launch_bounds__(32 * kGW) k_gsline(LevelView<T> L, int parity,
     const int chunks = (n + kGR - 1) / kGR;
     const size_t lim = (size_t)n * p;
     // the coefficients and the right-hand side of rows i0 .. i0 + kGR - 1 into val[b]
+    // (every load of a warp's rows is issued before the first is used; a row past the last is the last)
     auto form = [&](int k, int b) {
-        for (int r = warp - 1; r < kGR; r += kGW - 1) {
-            const int i = k * kGR + r;
-            if (i >= n) break;
-            const size_t o = (size_t)i * p + jc;
-            const bool hS = i + 1 < n, hN = i > 0;
-            const T gc = __ldg(L.G + o);
-            const T aS = face(gc, hS ? __ldg(L.G + o + p) : T(0), hS), aN = face(gc, hN ? __ldg(L.G + o - p) : T(0), hN);
-            const T aE = face(gc, hE ? __ldg(L.G + o + 1) : T(0), hE), aW = face(gc, hW ? __ldg(L.G + o - 1) : T(0), hW);
-            const T uE = hE ? __ldg(L.u + o + 1) : __ldg(L.u + o), uW = hW ? __ldg(L.u + o - 1) : __ldg(L.u + o);
+        const int r0 = (warp - 1) * kFR, i0 = k * kGR + r0;
+        if (i0 >= n) return;
+        T g[kFR + 2], gE[kFR], gW[kFR], uE[kFR], uW[kFR], f[kFR];
+        const size_t eE = hE ? 1 : 0, eW = hW ? 1 : 0;
+        g[0] = __ldg(L.G + (size_t)max(i0 - 1, 0) * p + jc);
+        g[kFR + 1] = __ldg(L.G + (size_t)min(i0 + kFR, n - 1) * p + jc);
+#pragma unroll
+        for (int r = 0; r < kFR; ++r) {
+            const size_t o = (size_t)min(i0 + r, n - 1) * p + jc;
+            g[r + 1] = __ldg(L.G + o);
+            gE[r] = __ldg(L.G + o + eE);
+            gW[r] = __ldg(L.G + o - eW);
+            uE[r] = __ldg(L.u + o + eE);
+            uW[r] = __ldg(L.u + o - eW);
+            f[r] = __ldg(L.f + o);
+        }
+#pragma unroll
+        for (int r = 0; r < kFR; ++r) {
+            const bool hS = i0 + r + 1 < n, hN = i0 + r > 0;
+            const T aS = face(g[r + 1], g[r + 2], hS), aN = face(g[r + 1], g[r], hN);
+            const T aE = face(g[r + 1], gE[r], hE), aW = face(g[r + 1], gW[r], hW);
             const T sum = add_rn(add_rn(aN, aS), add_rn(aE, aW));
-            const T across = fma_rn(aW, uW, mul_rn(aE, uE));
-            val[b][0][r][lane] = mul_rn(L.cdiff, aN);
-            val[b][1][r][lane] = mul_rn(L.cdiff, aS);
-            val[b][2][r][lane] = -fma_rn(L.cdiff, sum, L.inv_tau);
-            val[b][3][r][lane] = fma_rn(-L.cdiff, across, __ldg(L.f + o));
+            const T across = fma_rn(aW, uW[r], mul_rn(aE, uE[r]));
+            val[b][0][r0 + r][lane] = mul_rn(L.cdiff, aN);
+            val[b][1][r0 + r][lane] = mul_rn(L.cdiff, aS);
+            val[b][2][r0 + r][lane] = -fma_rn(L.cdiff, sum, L.inv_tau);
+            val[b][3][r0 + r][lane] = fma_rn(-L.cdiff, across, f[r]);
         }
     };
     // ---- elimination, downwards
@@ -108,14 +123,22 @@ __global__ void __launch_bounds__(32 * kGW) k_gsline(LevelView<T> L, int parity,
     }
     // ---- substitution, upwards: chunk k from its last row
     auto fetch = [&](int k, int b) {
-        for (int r = warp - 1; r < kGR; r += kGW - 1) {
-            const int i = k * kGR + r;
-            if (i >= n) break;
-            const size_t o = (size_t)i * p + jc, q = (size_t)i * p + (on ? c : 0);
-            const bool hS = i + 1 < n;
-            val[b][0][r][lane] = hS ? mul_rn(L.cdiff, face(__ldg(L.G + o), __ldg(L.G + o + p), true)) : T(0);
-            val[b][1][r][lane] = dg[q];
-            val[b][2][r][lane] = rg[q];
+        const int r0 = (warp - 1) * kFR, i0 = k * kGR + r0;
+        if (i0 >= n) return;
+        T g[kFR + 1], rec[kFR], rh[kFR];
+        g[kFR] = __ldg(L.G + (size_t)min(i0 + kFR, n - 1) * p + jc);
+#pragma unroll
+        for (int r = 0; r < kFR; ++r) {
+            const size_t row = (size_t)min(i0 + r, n - 1) * p, q = row + (on ? c : 0);
+            g[r] = __ldg(L.G + row + jc);
+            rec[r] = dg[q];
+            rh[r] = rg[q];
+        }
+#pragma unroll
+        for (int r = 0; r < kFR; ++r) {
+            val[b][0][r0 + r][lane] = i0 + r + 1 < n ? mul_rn(L.cdiff, face(g[r], g[r + 1], true)) : T(0);
+            val[b][1][r0 + r][lane] = rec[r];
+            val[b][2][r0 + r][lane] = rh[r];
         }
     };
     if (warp > 0) fetch(chunks - 1, (chunks - 1) & 1);
