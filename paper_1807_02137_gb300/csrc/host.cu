@@ -271,6 +271,8 @@ struct Solver final : SolverBase {
     int learn_skip = 0, learn_backoff = 1;   // plain V-cycles left before the next learned try
     long long learned_acc = 0, learned_rej = 0;
     size_t lb_smem = 0;
+    int lt = -1;                  // first grid of the tail kernel, where no bottom kernel applies (-1: not used)
+    size_t lt_smem = 0;
     int lb_pad = 0, lc_pad = 0;   // odd row pitches in the bottom kernels' shared memory
     ModelParams mp{};
 
@@ -499,6 +501,7 @@ struct Solver final : SolverBase {
         lb = lb_first = -1;
         lb_smem = 0;
         lc = -1;   // an explicit choice of the one-block bottom (or none) replaces the cluster
+        lt = -1;
         if (sizeof(T) == 4 && p.model == MG_MODEL_SC && fused()) {
             int ns[kMaxLevels], ms[kMaxLevels];
             for (int l = 0; l < nlev; ++l) { ns[l] = lv[l].n; ms[l] = lv[l].m; }
@@ -512,6 +515,16 @@ struct Solver final : SolverBase {
             int l = lb_first;
             while (l < nlev - 2 && lv[l].n * lv[l].m > kBottomThreads) ++l;
             use_bottom_from(lv[l].n * lv[l].m <= kBottomThreads ? l : lb_first);
+        }
+        if (enable && lb_first < 0 && fused() && p.nu1 >= 1 && p.nu2 >= 1) {   // the largest grid it takes
+            int ns[kMaxLevels], ms[kMaxLevels];
+            for (int l = 0; l < nlev; ++l) { ns[l] = lv[l].n; ms[l] = lv[l].m; }
+            for (int l = nlev - 2; l >= 1; --l) {
+                const size_t b = tail_smem_bytes<T>(ns, ms, l, nlev, p.precision == MG_MIXED);
+                if (!b) break;
+                lt = l;
+                lt_smem = b;
+            }
         }
         drop_graphs();
         return lb;
@@ -622,6 +635,26 @@ struct Solver final : SolverBase {
             if (cluster) launch_cluster(a, lc_tiles, lc_smem, st);
             else launch_bottom(a, lb_smem, st);
         }
+    }
+
+    // The tail kernel's first grid in the V-cycle being enqueued (relaxation weights: per-grid kernels).
+    int tail_level() const { return use_omega ? -1 : lt; }
+
+    void launch_tail_cycle(bool fas) {
+        TailArgs<T> a{};
+        a.first = lt; a.L = nlev; a.nu1 = p.nu1; a.nu2 = p.nu2;
+        a.fas = fas;
+        a.coarse_aos = p.coarse_solver == MG_COARSE_AOS;
+        a.coarse_maxit = p.coarse_maxit;
+        a.aos_dt = p.aos_dt;
+        a.coarse_tol = p.coarse_tol;
+        a.mp = mp;
+        a.sc = dsc;
+        for (int l = lt; l < nlev; ++l) {
+            a.g[l] = view(l);
+            a.h2nm[l] = h2nm(l);
+        }
+        launch_tail<T>(a, p.precision == MG_MIXED, lt_smem, st);
     }
 
     int reset(const void *image, const double *mk, int k) override {
@@ -872,6 +905,12 @@ struct Solver final : SolverBase {
             ++launches;
             return;
         }
+        if (l == tail_level()) {
+            launch_tail_cycle(l == fas_level);
+            fas_level = -1;
+            ++launches;
+            return;
+        }
         if (l == nlev - 1) {
             launch_coarse_solve<T>(view(l), p.precision == MG_MIXED, mp, A1 / ((double)n * m), h2nm(l),
                                    p.coarse_maxit, p.coarse_tol, coarse, dsc, p.coarse_solver == MG_COARSE_AOS,
@@ -892,9 +931,10 @@ struct Solver final : SolverBase {
             launches += 3;
         }
         // FAS right-hand side on grid l+1: rhs += L(pn + u0).  FP32 storage with a pre-smoothing
-        // on grid l+1: its first snapshot completes it (fas_level), in the bottom kernels too;
-        // otherwise a residual launch here
-        const bool fas_in_snapshot = std::is_same<T, float>::value && p.nu1 >= 1 && l + 1 < nlev - 1;
+        // on grid l+1: its first snapshot completes it (fas_level), in the bottom kernels and the tail
+        // kernel too; otherwise a residual launch here
+        const bool fas_in_snapshot = p.nu1 >= 1 && l + 1 < nlev - 1 &&
+                                     (std::is_same<T, float>::value || l + 1 == tail_level());
         if (fas_in_snapshot) {
             fas_level = l + 1;
             launches += area_launches(l);
@@ -2143,6 +2183,7 @@ int mg_setup(mg_handle *out, const void *image, int n, int m, const double *mark
     prepare_smoother_kernels();
     prepare_coarse_kernels();
     prepare_bottom_kernel();
+    prepare_tail_kernel();
     prepare_sweep_tma();
     prepare_snapshot_tma();
     prepare_residual_tma();
@@ -2548,6 +2589,7 @@ int mg_batch_setup(mg_batch *out, int count, const void *const *images, const in
     prepare_smoother_kernels();
     prepare_coarse_kernels();
     prepare_bottom_kernel();
+    prepare_tail_kernel();
     prepare_sweep_tma();
     prepare_snapshot_tma();
     prepare_residual_tma();

@@ -316,4 +316,22 @@ size_t cluster_smem_bytes(size_t bottom_bytes);
 int cluster_fits(int tiles, size_t smem);
 void launch_cluster(const BottomArgs &A, int tiles, size_t smem, cudaStream_t st);
 
+// tail_kernel.cu: grids first .. L-1 of a V-cycle in one block where bottom_kernel.cu does not apply (FP64
+// storage, the Rada-Chen model).  nu1 and nu2 are at least 1; fas as in BottomArgs.
+template <typename T>
+struct TailArgs {
+    int first, L, nu1, nu2, fas, coarse_aos, coarse_maxit;
+    double aos_dt, coarse_tol;
+    double h2nm[kMaxLevels];
+    ModelParams mp;
+    Scalars *sc;
+    LevelView<T> g[kMaxLevels];
+};
+constexpr size_t kTailSmemMax = 160 * 1024;
+template <typename T>
+size_t tail_smem_bytes(const int *n, const int *m, int first, int L, int coarse_fp64);   // 0: does not apply
+void prepare_tail_kernel();
+template <typename T>
+void launch_tail(const TailArgs<T> &A, int coarse_fp64, size_t smem, cudaStream_t st);
+
 }  // namespace segmg

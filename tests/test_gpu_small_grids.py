@@ -127,3 +127,30 @@ def test_batch_restart_rounds_equal_individual_solves(segmg):
             assert np.array_equal(b.solver(q).phi().cpu().numpy(), s.phi().cpu().numpy())
             s.close()
     b.close()
+
+
+# the tail kernel (one block for the smallest grids: FP64 storage, the Rada-Chen model) against the
+# per-grid kernels, down to what can be read of every grid; its first grid one cell wide of a limit,
+# long and thin, and as wide as it takes
+@pytest.mark.parametrize("kw", [{"precision": 1}, {"precision": 1, "model": 1}, {"model": 1},
+                                {"precision": 2, "model": 1}])
+@pytest.mark.parametrize("shape,levels,nu", [((130, 97), 6, (2, 2)), ((64, 64), 4, (1, 3)), ((33, 67), 5, (3, 1)),
+                                             ((20, 125), 4, (2, 1))])
+def test_tail_kernel_equals_per_grid_kernels(segmg, kw, shape, levels, nu):
+    names = {0: segmg.MG_F32, 1: segmg.MG_F64, 2: segmg.MG_MIXED}
+    par = {"precision": names[kw.get("precision", 0)], "model": segmg.MG_MODEL_RC if kw.get("model") else segmg.MG_MODEL_SC}
+    img, mk = image(*shape, 8)
+    outs, count = [], []
+    for on in (True, False):
+        s, p = gpu_solver(segmg, img, mk, levels=levels, nu1=nu[0], nu2=nu[1], **par)
+        s.set_bottom_kernel(on)
+        s.begin_step()
+        c0 = s.stats()["launches"]
+        rho = [s.vcycle() for _ in range(3)]
+        count.append(s.stats()["launches"] - c0)
+        outs.append([rho] + [s.level(l, f).cpu().numpy() for l in range(levels) for f in ("phi", "rhs", "G")
+                             if not (f == "G" and l == levels - 1) and not (f == "rhs" and l == 0)])
+        s.close()
+    assert count[0] < count[1]
+    for a, b in zip(*outs):
+        assert np.array_equal(a, b)
