@@ -6,7 +6,7 @@
 // the first grid that fits down to the coarsest and back, every grid in shared memory, with the
 // per-grid kernels' operations in their order (cell_G, face, point_relax, pcr_piece, the transfer
 // taps, the area sum's order, the coarsest solve): the results are the same numbers.  517x700 Rada-Chen
-// step 7.05 -> 6.17 ms, 128x128 FP64 step 29.4 -> 27.7 ms.
+// step 7.05 -> 5.97 ms, 128x128 FP64 step 29.4 -> 26.2 ms.
 //
 // First grid: at most 32 x 32 cells in FP32, one 32-cell piece a line and one area partial.  In FP64 at
 // most 256 cells: one SM does two FP64 multiply-adds a cycle, so a larger grid's cells cost more here
@@ -44,6 +44,7 @@ struct TailShared {
     uint8_t star[32][32];
     uint32_t mrow[2][32], mcol[2][32];   // member masks of the lines of sweeps A, B and C, D
     int s_err;
+    unsigned any;                        // bit k: sweep k has a member cell
 };
 
 // Cells (i, j) of an n x m grid (m <= 32): a power of two >= m threads a row.
@@ -103,6 +104,7 @@ __device__ __forceinline__ TFaces<T> t_faces(const TGrid<T> &B, int i, int j) {
 // Snapshot: G, f, the jump classes and the member masks.
 template <typename T>
 __device__ __forceinline__ void t_snapshot(const TGrid<T> &B, T ar, TailShared &S) {
+    if (threadIdx.x == 0) S.any = 0;
     t_G(B, B.u);
     const T *pn = sm<T>() + B.pn;
     const int n = B.n, m = B.m;
@@ -131,31 +133,36 @@ __device__ __forceinline__ void t_snapshot(const TGrid<T> &B, T ar, TailShared &
         const unsigned s = lane < m ? S.star[i][lane] : 0u;
         const uint32_t a = members_of(__ballot_sync(0xffffffffu, s & 1u), m);
         const uint32_t b = members_of(__ballot_sync(0xffffffffu, s & 2u), m);
-        if (lane == 0) { S.mrow[0][i] = a; S.mrow[1][i] = b; }
+        if (lane == 0) {
+            S.mrow[0][i] = a;
+            S.mrow[1][i] = b;
+            if (a | b) atomicOr(&S.any, (a ? 1u : 0u) | (b ? 2u : 0u));
+        }
     }
     for (int j = warp; j < m; j += kWarps) {
         const unsigned s = lane < n ? S.star[lane][j] : 0u;
         const uint32_t a = members_of(__ballot_sync(0xffffffffu, s & 4u), n);
         const uint32_t b = members_of(__ballot_sync(0xffffffffu, s & 8u), n);
-        if (lane == 0) { S.mcol[0][j] = a; S.mcol[1][j] = b; }
+        if (lane == 0) {
+            S.mcol[0][j] = a;
+            S.mcol[1][j] = b;
+            if (a | b) atomicOr(&S.any, (a ? 4u : 0u) | (b ? 8u : 0u));
+        }
     }
     __syncthreads();
 }
 
-// One directional sweep of Hybrid Smoother 2: two checkerboard phases, two partial-line phases (one
-// piece a line: nothing lies before or after it).
+// The two checkerboard phases of a sweep.
 template <typename T>
-__device__ __forceinline__ void t_sweep(const TGrid<T> &B, int sweep, TailShared &S) {
-    const int n = B.n, m = B.m;
-    const bool rev = sweep & 1, rowwise = sweep < 2;
+__device__ __forceinline__ void t_points(const TGrid<T> &B, int sweep, const TailShared &S) {
     T *u = sm<T>() + B.u;
     const T *f = sm<T>() + B.f;
 #pragma unroll 1
     for (int ph = 0; ph < 2; ++ph) {
-        const int colour = rev ? 1 - ph : ph;
-        TAIL_CELLS(n, m, i, j) {
+        const int colour = (sweep & 1) ? 1 - ph : ph;
+        TAIL_CELLS(B.n, B.m, i, j) {
             if (((i + j) & 1) != colour) continue;
-            const uint32_t mk = rowwise ? S.mrow[sweep][i] >> j : S.mcol[sweep - 2][j] >> i;
+            const uint32_t mk = sweep < 2 ? S.mrow[sweep][i] >> j : S.mcol[sweep - 2][j] >> i;
             if (mk & 1u) continue;
             const TFaces<T> a = t_faces(B, i, j);
             const int q = i * B.P + j;
@@ -163,6 +170,15 @@ __device__ __forceinline__ void t_sweep(const TGrid<T> &B, int sweep, TailShared
         }
         __syncthreads();
     }
+}
+
+// The two partial-line phases of a sweep (one piece a line: nothing lies before or after it).
+template <typename T>
+__device__ __forceinline__ void t_lines(const TGrid<T> &B, int sweep, const TailShared &S) {
+    const int n = B.n, m = B.m;
+    const bool rev = sweep & 1, rowwise = sweep < 2;
+    T *u = sm<T>() + B.u;
+    const T *f = sm<T>() + B.f;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nlines = rowwise ? n : m, len = rowwise ? m : n;
 #pragma unroll 1
@@ -184,6 +200,54 @@ __device__ __forceinline__ void t_sweep(const TGrid<T> &B, int sweep, TailShared
             if (pcr_piece<T>(mk, len, B.cdiff, B.inv_tau, own, T(0), T(0), at, x)) u[place(lane)] = x;
         }
         __syncthreads();
+    }
+}
+
+// The four sweeps of Hybrid Smoother 2 after the snapshot.  On a grid of one cell a thread the cell's
+// faces, diagonal, f and member bits stay in registers over all of them: FP64 face sums and diagonals
+// are then formed once, not in each of eight phases (128x128 FP64 step 27.6 -> 26.2 ms).  Line phases
+// without a member are skipped.
+template <typename T>
+__device__ __forceinline__ void t_sweeps(const TGrid<T> &B, const TailShared &S) {
+    const unsigned any = S.any;
+    const int lg = B.m <= 1 ? 0 : 32 - __clz(B.m - 1), i = (int)threadIdx.x >> lg, j = (int)threadIdx.x & ((1 << lg) - 1);
+    if (B.n > kNT >> lg) {
+#pragma unroll 1
+        for (int k = 0; k < 4; ++k) {
+            t_points(B, k, S);
+            if ((any >> k) & 1u) t_lines(B, k, S);
+        }
+        return;
+    }
+    const bool own = i < B.n && j < B.m;
+    T *u = sm<T>() + B.u;
+    TFaces<T> a{};
+    T dv = T(1), fq = T(0);
+    int q = 0, colour = 2;
+    unsigned mem = 0;
+    if (own) {
+        a = t_faces(B, i, j);
+        q = i * B.P + j;
+        dv = fma_rn(B.cdiff, add_rn(add_rn(a.S, a.N), add_rn(a.E, a.W)), B.inv_tau);
+        fq = sm<T>()[B.f + q];
+        colour = (i + j) & 1;
+        mem = ((S.mrow[0][i] >> j) & 1u) | (((S.mrow[1][i] >> j) & 1u) << 1) | (((S.mcol[0][j] >> i) & 1u) << 2) |
+              (((S.mcol[1][j] >> i) & 1u) << 3);
+    }
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll 1
+        for (int ph = 0; ph < 2; ++ph) {
+            if (colour == (ph ^ (k & 1)) && !((mem >> k) & 1u)) {
+                T num = mul_rn(a.S, u[a.oS]);
+                num = fma_rn(a.N, u[a.oN], num);
+                num = fma_rn(a.E, u[a.oE], num);
+                num = fma_rn(a.W, u[a.oW], num);
+                u[q] = div_relax(fma_rn(B.cdiff, num, -fq), dv);
+            }
+            __syncthreads();
+        }
+        if ((any >> k) & 1u) t_lines(B, k, S);
     }
 }
 
@@ -344,8 +408,7 @@ __global__ void __launch_bounds__(kNT) k_tail(const __grid_constant__ TailArgs<T
                 fas = false;
             }
             t_snapshot(B, ar, S);
-#pragma unroll 1
-            for (int k = 0; k < 4; ++k) t_sweep(B, k, S);
+            t_sweeps(B, S);
             ++t;
         } else if (down) {
             t_residual(B, B.u, B.f, 0, rc ? t_area(B, B.u, A.mp, A1frac, S.red) : T(0));
