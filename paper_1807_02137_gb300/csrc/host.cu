@@ -678,12 +678,11 @@ struct Solver final : SolverBase {
         double s = 0;
         for (int t = -R; t <= R; ++t) { taps[t + R] = std::exp(-(double)t * t / (2 * p.sigma_blur * p.sigma_blur)); s += taps[t + R]; }
         for (double &t : taps) t /= s;
-        launch_blur<T>(L0.z, L0.G, L0.f, n, m, L0.pitch, L0.pitch, taps.data(), R, st);
         // markers, hull and the initial area go through pinned staging (asynchronous copies)
         double *smk = hstage, *shull = hstage + 2 * kcap, *sA1 = hstage + 6 * kcap + 8;
         std::memcpy(smk, mk, sizeof(double) * 2 * k);
         CK(cudaMemcpyAsync(dmk, smk, sizeof(double) * 2 * k, cudaMemcpyHostToDevice, st));
-        launch_edge_distance<T>(L0.f, L0.w, L0.d, n, m, L0.pitch, p.beta_edge, dmk, k, p.sigma_d, p.model, st);
+        launch_image_weights<T>(L0.z, L0.w, L0.d, n, m, L0.pitch, taps.data(), R, p.beta_edge, dmk, k, p.sigma_d, p.model, st);
         for (int l = 1; l < nlev; ++l) {
             Level<T> &Pf = lv[l - 1], &Lc = lv[l];
             RestrictFields<T> F{};
@@ -720,8 +719,8 @@ struct Solver final : SolverBase {
         *sA1 = area / ((double)n * m);
         CK(cudaMemcpyAsync(&dsc->A1frac, sA1, sizeof(double), cudaMemcpyHostToDevice, st));
         launch_region_sums<T>(view(0), p.eps, partials, npart, dsc, 1, st);
-        // copy-in, two blur passes, edge / distance, initial phi, region sums (2), restrictions
-        launches += 5 + norm_launches() + (nlev - 1) + (p.precision == MG_MIXED ? nlev : 0);
+        // copy-in, weights, initial phi, region sums (2), restrictions
+        launches += 3 + norm_launches() + (nlev - 1) + (p.precision == MG_MIXED ? nlev : 0);
         CKL();
         CK(cudaMemcpyAsync(hsc, dsc, sizeof(Scalars), cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));   // the staging buffer is free again; the image's check

@@ -98,10 +98,7 @@ __device__ __forceinline__ T weight_at(const LevelView<T> &L, size_t o) {
 
 // setup_kernels.cu
 template <typename T>
-void launch_blur(const T *src, T *tmp, T *dst, int n, int m, int pitch_src, int pitch, const double *taps,
-                 int R, cudaStream_t st);
-template <typename T>
-void launch_edge_distance(const T *zb, T *w, T *d, int n, int m, int pitch, double beta_edge,
+void launch_image_weights(const T *z, T *w, T *d, int n, int m, int pitch, const double *taps, int R, double beta_edge,
                           const double *mk, int k, double sigma_d, int model, cudaStream_t st);
 // The n x m image (row-major, no padding) into the pitched finest z; bit 2 of *flag is set
 // when a value is NaN or Inf.

@@ -154,3 +154,26 @@ def test_tail_kernel_equals_per_grid_kernels(segmg, kw, shape, levels, nu):
     assert count[0] < count[1]
     for a, b in zip(*outs):
         assert np.array_equal(a, b)
+
+
+# set-up and step start on 32 x 32 tiles: single rows and columns, one beside a tile edge, grids
+# narrower than the blur's reach (sigma 1: 3, sigma 5: 15 cells), more markers than a chunk of 32
+@pytest.mark.parametrize("shape,sigma,k", [((1, 40), 1.0, 3), ((33, 31), 1.0, 5), ((2, 65), 5.0, 4), ((70, 3), 5.0, 3),
+                                           ((97, 130), 2.0, 70)])
+@pytest.mark.parametrize("model", [0, 1])
+def test_setup_tiles_match_oracle(segmg, shape, sigma, k, model):
+    n, m = shape
+    rng = np.random.default_rng(n + m)
+    img = rng.random((n, m))
+    mk = np.stack([rng.uniform(0, m - 1, k), rng.uniform(0, n - 1, k)], axis=1)
+    s, p = gpu_solver(segmg, img, mk, precision=segmg.MG_F64, levels=1 if min(shape) < 4 else 2, sigma_blur=sigma,
+                      model=model)
+    o = O.Solver(img, mk, oracle_params(n, m, p))
+    s.begin_step(); o.begin_step()
+    for f in ("w", "z", "d"):
+        assert relmax(s.level(0, f).cpu().numpy(), o.level(0, f)) < 1e-13, f
+    assert relmax(s.phi().cpu().numpy(), o.phi) < 1e-13
+    F = s.level(0, "F").cpu().numpy() - s.phi().cpu().numpy() / p.tau
+    assert relmax(F, o.level(0, "Fn")) < 1e-12
+    assert np.array_equal(s.mask().cpu().numpy() > 0, s.phi().cpu().numpy() > 0)
+    s.close(); o.close()
