@@ -196,6 +196,10 @@ __device__ __forceinline__ void cp_async_elem(T *smem, const T *gmem, bool pred)
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
+template <typename T> struct Pair;   // two neighbouring values
+template <> struct Pair<float> { using type = float2; };
+template <> struct Pair<double> { using type = double2; };
+
 template <typename T> struct VecOf;
 template <> struct VecOf<float> { using type = float4; static constexpr int n = 4; };
 template <> struct VecOf<double> { using type = double2; static constexpr int n = 2; };

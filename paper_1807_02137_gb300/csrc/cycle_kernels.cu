@@ -271,26 +271,42 @@ __global__ void __launch_bounds__(256) k_sum_partials(const double *partials, in
     if (threadIdx.x == 0) *out = s;
 }
 
-// Full weighting of up to three fields of one grid in one launch (blockIdx.z picks the field).
+// Full weighting of up to three fields of one grid in one launch (blockIdx.z picks the field): three
+// taps per axis, or two of weight 1/2 at the last coarse cell of an even axis (fw_taps).  Everything is
+// read through L2 (see tma.cuh): a lane reads its two fine columns of a row as one vector and takes the
+// third from the next lane, three loads for nine (three fields of 8192^2 0.559 -> 0.519 ms; what is left
+// is the lifetime of blocks with one cell a thread).
 template <typename T>
 __global__ void __launch_bounds__(256) k_restrict(RestrictFields<T> F, int n, int m, int pf, int pc) {
+    using V2 = typename Pair<T>::type;
     const int J = blockIdx.x * 32 + threadIdx.x, I = blockIdx.y * 8 + threadIdx.y;
     const int nc = n / 2, mc = m / 2;
     pdl_wait();
     pdl_trigger();
-    if (I >= nc || J >= mc) return;
+    if (I >= nc) return;   // the whole warp
     const T *f = F.f[blockIdx.z];
     T *c = F.c[blockIdx.z], *c2 = F.c2[blockIdx.z];
-    int ri[3], ci[3];
-    float rw[3], cw[3];
-    int nr = fw_taps(I, n, ri, rw), nk = fw_taps(J, m, ci, cw);
-    T s = T(0);
-    for (int a = 0; a < nr; ++a) {
-        T row = T(0);
-        for (int b = 0; b < nk; ++b)
-            row = fma_rn(T(cw[b]), ldl2(f, (size_t)ri[a] * pf + ci[b], (size_t)n * pf, kDbgResidual), row);
-        s = fma_rn(T(rw[a]), row, s);
+    const int Jc = min(J, mc - 1);   // a lane past the last column repeats it
+    const bool r3 = 2 * I + 2 < n, c3 = 2 * Jc + 2 < m, edge = threadIdx.x == 31 || Jc == mc - 1;
+    const size_t lim = (size_t)n * pf;
+    V2 v[3];
+    T third[3] = {T(0), T(0), T(0)};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const size_t o = (size_t)(2 * I + (a == 2 && !r3 ? 1 : a)) * pf + 2 * Jc;
+        v[a] = MG_DBG_OK(o + 1, lim, kDbgResidual) ? __ldcg(reinterpret_cast<const V2 *>(f + o)) : V2{};
+        if (edge && c3) third[a] = ldl2(f, o + 2, lim, kDbgResidual);
     }
+    const T rw = r3 ? T(0.25) : T(0.5), cw = c3 ? T(0.25) : T(0.5);
+    T s = T(0);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const T next = __shfl_down_sync(0xffffffffu, v[a].x, 1);
+        T row = fma_rn(T(0.5), v[a].y, fma_rn(cw, v[a].x, T(0)));
+        if (c3) row = fma_rn(cw, edge ? third[a] : next, row);
+        if (a < 2 || r3) s = fma_rn(a == 1 ? T(0.5) : rw, row, s);
+    }
+    if (J >= mc) return;
     stc(c, (size_t)I * pc + J, (size_t)nc * pc, kDbgResidual, s);
     if (c2) stc(c2, (size_t)I * pc + J, (size_t)nc * pc, kDbgResidual, s);
 }
