@@ -369,6 +369,9 @@ int mg_energy(mg_handle h, double *E);
  * set-up the cluster bottom kernel (mg_set_cluster_level) is also chosen, from the largest grid
  * the one-block kernel can start at, when that grid has at most 16 tiles of 32 x 32 and such a
  * cluster fits the GPU; this call and mg_set_bottom_level switch the cluster off.
+ * Where neither applies (MG_F64, the Rada-Chen model; fused smoother, nu1 and nu2 >= 1, no relaxation
+ * weights) a one-block kernel runs the smallest grids with the per-grid kernels' operations; it is not
+ * reported in mg_stats, and enable = 0 switches it off.
  * Errors: MG_ERR_ARG. */
 int mg_set_bottom_kernel(mg_handle h, int enable, int *first_level);
 /* Sets the first grid of the one-block bottom kernel (a tuning step of this implementation; the
