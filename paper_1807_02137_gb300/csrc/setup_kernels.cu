@@ -443,8 +443,9 @@ void launch_image_weights(const T *z, T *w, T *d, int n, int m, int pitch, const
     for (int t = 0; t <= 2 * R && t < 33; ++t) tp.w[t] = T(taps[t]);
     const T inv_s2 = T(1.0 / (2.0 * sigma_d * sigma_d));
     const size_t smem = image_weights_smem<T>(R);
-    if (smem + 2 * sizeof(T) * kMarkChunk * 32 > 48 * 1024)   // FP64 and a wide blur
-        cudaFuncSetAttribute(k_image_weights<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem + 2 * sizeof(T) * kMarkChunk * 32 > 48 * 1024)   // FP64 and a wide blur: room for the widest
+        cudaFuncSetAttribute(k_image_weights<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)image_weights_smem<T>(16));
     k_image_weights<T><<<dim3((m + 31) / 32, (n + 31) / 32), dim3(32, 8), smem, st>>>(z, w, d, n, m, pitch, tp, R,
                                                                                     T(beta_edge), mk, k, inv_s2, model);
 }
